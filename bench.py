@@ -133,10 +133,9 @@ DFT_FLOPS = {1: 0, 2: 4, 3: 18, 4: 16, 5: 52, 6: 48, 7: 102, 8: 60, 10: 124, 12:
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12     # SMs x FP32 lanes x FMA x max SM clock
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of the same
-# kernels: pass 2 on the full 512-pair launch at 96^3 (a one-pass metric set), per line
-# split and CTA size (8 lanes x 2A at 256 threads: 3.669 + 3.602 GB); the SYRK on a small
-# case scaled by the panel bytes it reads
-PASS2_DRAM_BYTES_PER_PAIR_96 = {(8, 256): 7.271e9 / 512}
+# kernels: pass 2 on the full 512-pair launch at 96^3 (a one-pass metric set: 3.669 + 3.602
+# GB); the SYRK on a small case scaled by the panel bytes it reads
+PASS2_DRAM_BYTES_PER_PAIR_96 = 7.271e9 / 512
 SYRK_DRAM_PER_PANEL_BYTE = 1.938e9 / 1.850e9    # DRAM bytes per byte of the two bf16 panels
 
 
@@ -144,7 +143,7 @@ def _modinv(a, m):
     return next(i for i in range(1, m + 1) if (a * i) % m == 1 % m)
 
 
-_PFA = {6: (2, 3), 10: (2, 5), 12: (3, 4), 14: (2, 7), 24: (3, 8)}
+_PFA = {6: (2, 3), 10: (2, 5), 12: (3, 4), 14: (2, 7), 20: (4, 5), 24: (3, 8), 28: (4, 7)}
 
 
 def _pfa_maps(A):
@@ -154,16 +153,20 @@ def _pfa_maps(A):
 
 
 def _small_in(m):
-    """P-point DFT (P = 2, 3) with the inputs flagged False zero (all outputs formed)."""
+    """P-point DFT (P = 2, 3, 4) with the inputs flagged False zero (all outputs formed)."""
     n = sum(m)
+    if len(m) == 4:
+        return 8    # two adjacent inputs
     if len(m) == 2:
         return 4 if n == 2 else 0
     return DFT_FLOPS[3] if n == 3 else 12 if n == 2 else (0 if m[0] else 8)
 
 
 def _small_out(w):
-    """P-point DFT (P = 2, 3) forming only the outputs flagged True."""
+    """P-point DFT (P = 2, 3, 4) forming only the outputs flagged True."""
     n = sum(w)
+    if len(w) == 4:
+        return 8 + 2 * n
     if len(w) == 2:
         return 4 if n == 2 else 2 * n
     if n == 0:
@@ -218,15 +221,19 @@ def line_flops_l8(A, kind):
     raise ValueError(kind)
 
 
-def algorithmic_flops(kernel, shape, nq, npsi_out, lanes=16):
-    """Implemented FP32 flops of one launch over nq pairs (npsi_out outputs for pass 3);
-    lanes: the line split of pass 2 (16 x A or 8 x 2A)."""
+def pass2_lanes(edge):
+    """Lanes per line of the FP32 y/z pass: 8 (x 2A), 16 (x A) at edge 112."""
+    return 16 if edge == 112 else 8
+
+
+def algorithmic_flops(kernel, shape, nq, npsi_out):
+    """Implemented FP32 flops of one launch over nq pairs (npsi_out outputs for pass 3)."""
     nz, ny, nx = shape
     Ax, Ay, Az = nx // 8, ny // 8, nz // 8
     Hx = nx + 1
     if kernel == "pass2_yz_kernel":
         Ly = 16 * Ay
-        lf = line_flops_l8 if lanes == 8 else line_flops
+        lf = line_flops_l8 if pass2_lanes(nz) == 8 else line_flops
         plane = (nz * lf(Ay, "fwd_pruned")
                  + Ly * (lf(Az, "fwd_pruned") + 2 * 16 * Az + lf(Az, "z_inverse"))
                  + nz * lf(Ay, "inv_keep_half"))
@@ -335,20 +342,18 @@ def run_rsx(args, rank, local_rank, world):
         # report the ALU roofline, with the HBM view alongside
         byts = [algorithmic_bytes(top, shape, nq, NOCC, NPSI if nq == SOLVES_EXCHANGE else 0)
                 for nq in per_launch_pairs[top]]
-        lanes = (tuning or {}).get("p2_lanes", 8 if os.environ.get("RSX_PASS2_LANES") == "8" else 16)
-        p2_threads = (tuning or {}).get("p2_threads", int(os.environ.get("RSX_PASS2_THREADS", "256")))
-        flops = [algorithmic_flops(top, shape, nq, 0, lanes) for nq in per_launch_pairs[top]]
+        flops = [algorithmic_flops(top, shape, nq, 0) for nq in per_launch_pairs[top]]
         avg_bytes = sum(byts) / len(byts)
         avg_flops = sum(flops) / len(flops)
         avg_ms = kernels[top]["ms_per_launch"]
         ach_f = avg_flops / (avg_ms / 1e3) / 1e12
         ach_b = avg_bytes / (avg_ms / 1e3) / 1e9
         traffic = None
-        per_pair = PASS2_DRAM_BYTES_PER_PAIR_96.get((lanes, p2_threads))
+        per_pair = PASS2_DRAM_BYTES_PER_PAIR_96
         if top == "pass2_yz_kernel" and tuple(shape) == (96, 96, 96) and per_pair:
             traffic = per_pair * sum(per_launch_pairs[top]) / len(per_launch_pairs[top])
-        split = "8 lanes x 2A" if lanes == 8 else "16 lanes x A"
-        roof = {"kernel": f"{top} ({split}, {p2_threads} threads)", "bound": "alu", "achieved": round(ach_f, 2),
+        split = "8 lanes x 2A" if pass2_lanes(shape[0]) == 8 else "16 lanes x A"
+        roof = {"kernel": f"{top} ({split})", "bound": "alu", "achieved": round(ach_f, 2),
                 "peak": round(FP32_PEAK_TFLOPS, 2),
                 "unit": "TFLOP/s", "frac": round(ach_f / FP32_PEAK_TFLOPS, 4), "traffic": traffic,
                 "traffic_source": (f"ncu DRAM bytes of the 512-pair launch ({per_pair / 1e6:.1f} MB per pair) times "

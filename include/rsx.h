@@ -74,21 +74,16 @@ const char* rsx_last_error(const rsx_ctx* ctx);
 int rsx_set_workspace_limit(rsx_ctx* ctx, size_t bytes);
 
 /* Tuning knobs of the pair-solve path (performance only: the results stay bitwise
- * identical under every knob except p2_lanes, which changes the rounding order of the
- * line transforms, both splits being equally accurate).
- *   p2_threads     threads per CTA of the y/z transform pass: 256, 384 (FP32) or 512; a
- *                  size is used only where its line scratch and the work plane fit in
- *                  shared memory (else 256)
+ * identical under every knob).
+ *   p2_threads     256, 384 or 512: kept for callers that set it; the y/z transform pass has
+ *                  one CTA size per box edge and precision, so it chooses nothing
  *   chunk_outputs  output orbitals per exchange chunk (0 = as many as the workspace holds)
  *   p1_group       x-pass block order: 0 pair-major, G > 0 pairs fastest in groups of G
  *   p2_global      1: the y/z pass keeps its work plane in a global (L2-resident) scratch
  *                  slice per CTA even where shared memory would hold it; 0: shared memory
  *                  whenever it fits
- *   p2_lanes       radix split of the y/z line transforms, M = 2n points per line: 16 (16
- *                  lanes x A: A-point DFTs in registers, then 16-point DFTs across lanes)
- *                  or 8 (8 lanes x 2A: 2A-point DFTs, then 8-point DFTs; FP32 with
- *                  shared-memory plane and A = M / 16 in {4, 8, 12}, i.e. edges 32, 64, 96;
- *                  elsewhere the 16-lane split runs) */
+ *   p2_lanes       16 or 8: kept for callers that set it; the line split of the y/z pass is
+ *                  8 lanes x M / 8 points (16 lanes x M / 16 in FP32 at edge 112) */
 typedef struct rsx_tuning {
   int p2_threads;
   int chunk_outputs;
@@ -101,10 +96,8 @@ int rsx_get_tuning(rsx_ctx* ctx, rsx_tuning* out);
 int rsx_set_tuning_ex(rsx_ctx* ctx, const rsx_tuning* t);
 /* Autotuner (the paper has no counterpart; a performance knob).  Times the exchange
  * apply for nocc x npsi pairs on synthetic device data under candidate knobs, by
- * coordinate descent from the current ones: pass-2 CTA size x plane staging x line split
- * (16 or 8 lanes), then the pass-1 block order (0, 4, 16, 64, all), then output orbitals
- * per chunk (1, 2, 4, all);
- * applies the fastest to the context.  With a non-empty cache_path the result is appended
+ * coordinate descent from the current ones: the pass-1 block order (0, 4, 16, 64, all), then
+ * output orbitals per chunk (1, 2, 4, all); applies the fastest to the context.  With a non-empty cache_path the result is appended
  * to that text file, keyed by box, precision, nocc, npsi, SM count and device name, and a
  * later call with the same key applies it without timing.  chosen (may be NULL) receives
  * the knobs, best_ms the best time (-1 if taken from the cache).  Synchronises the device.

@@ -9,6 +9,7 @@
 #include "../../include/rsx.h"
 #include "api_internal.cuh"
 #include "dense.cuh"
+#include "poisson_pass2.cuh"
 
 using namespace rsx;
 
@@ -153,31 +154,23 @@ int make_tables(rsx_ctx* c) {
   const double npad = (double)g.Mz * g.My * g.Mx;
   const double scale = c->h * c->h * c->h / npad;
   cudaError_t e = launch_ghat(g, c->h, scale, dcos[0], dcos[1], dcos[2], b0, b1, c->vhat, sizeof(R) == 8, 0);
-  if (e == cudaSuccess && sizeof(R) == 4) {
-    size_t hz_have = 0;
-    if (grow(c, &c->vhatz, &hz_have, (size_t)hx * hy * g.Mz * sizeof(float), "kernel table (lane order)") != RSX_OK)
-      e = cudaErrorMemoryAllocation;
-    else
-      e = launch_vhat_lanes(g, (const float*)c->vhat, (float*)c->vhatz, 0);
-  }
-  if (e == cudaSuccess && sizeof(R) == 4 && g.Ay == g.Az && g.Ay % 4 == 0) {
-    // the 8-lane y/z kernel: its lane-order table and twiddles w_M^{-t k1}, t < 8, k1 < 2 A
-    size_t have8 = 0, have_tw = 0;
-    const int A2 = 2 * g.Az;
-    std::vector<Cx<float>> tw8(8 * A2);
-    for (int t = 0; t < 8; ++t)
-      for (int k1 = 0; k1 < A2; ++k1) {
-        const long long ex = (long long)t * k1 % g.Mz;
-        const double ang = 2.0 * M_PI * (double)ex / (double)g.Mz;
-        tw8[t * A2 + k1].x = (float)cos(ang);
-        tw8[t * A2 + k1].y = (float)(-sin(ang));
+  if (e == cudaSuccess) {
+    // the y/z pass: its lane-order table and twiddles w_M^{-t k1}, t < lanes, k1 < M / lanes
+    size_t have_vl = 0, have_tw = 0;
+    const int lanes = p2_lanes<R>(g.Az), rad = g.Mz / lanes;
+    std::vector<Cx<R>> twl(g.Mz);
+    for (int t = 0; t < lanes; ++t)
+      for (int k1 = 0; k1 < rad; ++k1) {
+        const double ang = 2.0 * M_PI * (double)(t * k1) / (double)g.Mz;
+        twl[t * rad + k1].x = (R)cos(ang);
+        twl[t * rad + k1].y = (R)(-sin(ang));
       }
-    if (grow(c, &c->vhatz8, &have8, (size_t)hx * hy * g.Mz * sizeof(float), "kernel table (8-lane order)") != RSX_OK ||
-        grow(c, &c->tw8, &have_tw, tw8.size() * sizeof(Cx<float>), "8-lane twiddles") != RSX_OK)
+    if (grow(c, &c->vlanes, &have_vl, (size_t)hx * hy * p2_row_factors<R>(g.Az) * sizeof(R), "kernel table (lane order)") != RSX_OK ||
+        grow(c, &c->twl, &have_tw, twl.size() * sizeof(Cx<R>), "line twiddles") != RSX_OK)
       e = cudaErrorMemoryAllocation;
     else
-      e = cudaMemcpy(c->tw8, tw8.data(), tw8.size() * sizeof(Cx<float>), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = launch_vhat_lanes8(g, (const float*)c->vhat, (float*)c->vhatz8, 0);
+      e = cudaMemcpy(c->twl, twl.data(), twl.size() * sizeof(Cx<R>), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = launch_vhat_lanes<R>(g, (const R*)c->vhat, (R*)c->vlanes, 0);
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   cudaFree(b0);
@@ -219,8 +212,6 @@ int solve_pairs(rsx_ctx* c, const PairMap<R>& pm, int q0, int nq, int p0, int np
   int rc = grow(c, &c->work, &c->work_bytes, need, "FFT intermediates");
   if (rc) return rc;
   Cx<R>* inter = (Cx<R>*)c->work;
-  const Cx<R>* twz = (const Cx<R>*)c->tw[0];
-  const Cx<R>* twy = (const Cx<R>*)c->tw[1];
   const Cx<R>* twx = (const Cx<R>*)c->tw[2];
   {
     ProfScope ps(c, kKPass1, s);
@@ -237,16 +228,13 @@ int solve_pairs(rsx_ctx* c, const PairMap<R>& pm, int q0, int nq, int p0, int np
     grid = (int)std::min<long long>(nwork, (long long)per_sm * c->nsm);
   } else {
     grid = (int)std::min<long long>(nwork, 2LL * c->nsm);
-    const size_t gneed = (size_t)grid * g.nz * (g.My + 1) * sizeof(Cx<R>);
-    rc = grow(c, &c->gscr, &c->gscr_bytes, gneed, "pass-2 plane scratch");
+    rc = grow(c, &c->gscr, &c->gscr_bytes, pass2_gscratch_bytes<R>(g, grid), "pass-2 plane scratch");
     if (rc) return rc;
     gscr = (R*)c->gscr;
   }
   {
     ProfScope ps(c, kKPass2, s);
-    rc = check_cuda(c, launch_pass2<R>(g, nq, inter, twy, twz, (const R*)c->vhat, (const float*)c->vhatz, gscr, grid, s,
-                                       (const Cx<float>*)c->tw8, (const float*)c->vhatz8),
-                    "pass 2");
+    rc = check_cuda(c, launch_pass2<R>(g, nq, inter, (const Cx<R>*)c->twl, (const R*)c->vlanes, gscr, grid, s), "pass 2");
   }
   if (rc) return rc;
   if (out != nullptr) {
@@ -436,13 +424,9 @@ int rsx_create(rsx_ctx** out, int nz, int ny, int nx, double h, int precision, i
   g.Mz = 2 * nz; g.My = 2 * ny; g.Mx = 2 * nx;
   g.Az = g.Mz / 16; g.Ay = g.My / 16; g.Ax = g.Mx / 16;
   g.Hx = g.Mx / 2 + 1;
-  g.p2_threads = 256;
-  if (const char* e = getenv("RSX_PASS2_THREADS")) g.p2_threads = (atoi(e) == 512 || atoi(e) == 384) ? atoi(e) : 256;
   g.p1_group = 1 << 30;   // pass-1 blocks pair-fastest over the whole launch (orbital rows shared in L2)
   if (const char* e = getenv("RSX_PASS1_GROUP")) g.p1_group = atoi(e) > 0 ? atoi(e) : 0;
   g.p2_global = 0;
-  g.p2_lanes = 16;
-  if (const char* e = getenv("RSX_PASS2_LANES")) g.p2_lanes = atoi(e) == 8 ? 8 : 16;
   cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, device);
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
@@ -477,7 +461,7 @@ int rsx_destroy(rsx_ctx* c) {
   cudaDeviceSynchronize();
   prof_collect(c);
   for (cudaEvent_t e : c->prof_pool) cudaEventDestroy(e);
-  void* bufs[] = {c->vhat, c->vhatz, c->vhatz8, c->tw8, c->tw[0], c->tw[1], c->tw[2], c->work, c->gscr, c->dsm, c->smallr, c->status,
+  void* bufs[] = {c->vhat, c->vlanes, c->twl, c->tw[0], c->tw[1], c->tw[2], c->work, c->gscr, c->dsm, c->smallr, c->status,
                   c->panel_hi, c->panel_lo, c->gemm_part, c->eig_work, c->gscr_kd, c->pos, c->tdhf_work, c->specw, c->ones};
   for (void* b : bufs)
     if (b) cudaFree(b);

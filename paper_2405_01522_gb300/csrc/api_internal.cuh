@@ -27,9 +27,8 @@ struct rsx_ctx {
   size_t work_limit = 0;
   // device buffers owned by the context
   void* vhat = nullptr;                 // kernel table T[kx][ky][kz] (R)
-  void* vhatz = nullptr;                // FP32: the same in pass 2's lane order (launch_vhat_lanes)
-  void* vhatz8 = nullptr;               // FP32, Ay % 4 == 0: the order of the 8-lane y/z kernel
-  void* tw8 = nullptr;                  // FP32, Ay % 4 == 0: twiddles w_M^{-t k1}, t < 8, k1 < 2 Ay
+  void* vlanes = nullptr;               // the same in pass 2's lane order (R, launch_vhat_lanes)
+  void* twl = nullptr;                  // y/z line twiddles w_M^{-t k1}, t < lanes, k1 < M / lanes (R)
   void* tw[3] = {nullptr, nullptr, nullptr};
   void* work = nullptr;   size_t work_bytes = 0;     // FFT intermediates
   void* gscr = nullptr;   size_t gscr_bytes = 0;     // pass-2 planes when shared memory is too small
@@ -46,6 +45,7 @@ struct rsx_ctx {
   void* ones = nullptr; size_t ones_bytes = 0;           // unit field (R), Poisson solves of a density
   void* tdhf_work = nullptr; size_t tdhf_work_bytes = 0; // full TDHF: L, A + B, products
   int p2_occ[2] = {0, 0};
+  int p2_threads = 256, p2_lanes = 16;   // tuning knobs kept for callers (no effect, see rsx.h)
   int chunk_outputs = 0;   // tuning: output orbitals per exchange chunk (0 = as many as fit)
   long long wait_limit = -1;   // spin rounds of the bounded grid waits (-1: the kernels' default)
   // host-side fault injection (testing aid): fail the workspace allocation after

@@ -5,6 +5,7 @@
 #include <cstdint>
 
 #include "dense.cuh"
+#include "poisson_pass2.cuh"
 #include "tcgen05_util.cuh"
 #include "gemm_tcgen05.cuh"
 #include "../../include/rsx.h"
@@ -493,50 +494,37 @@ __global__ void k_pair_products(const R* __restrict__ A, int na, const R* __rest
   }
 }
 
-// Pass 2's FP32 copy of the kernel table in the order its lanes read it: after the
-// 16-point z transforms lane t (< Az) holds kz = t + Az k2, k2 < 16, and reads the
-// factors of one column (kx, |ky|) as four float4 at [(k2 / 4) Az + t], so that a
-// half-warp's request covers 16 contiguous bytes per lane.  out[kx][iy][k2/4][t][k2%4] =
-// T[kx][iy][fold(t + Az k2)], fold(kz) = min(kz, Mz - kz).
-__global__ void k_vhat_lanes(const float* __restrict__ T, int rows, int hz, int Az, float* __restrict__ out) {
-  const int Mz = 16 * Az;
-  const size_t n = (size_t)rows * Mz;
+// Pass 2's copy of the kernel table in the order its lanes read it (poisson_lines.cuh), as
+// consecutive values per lane and folded column (kx, |ky|).  8 lanes: lane s holds kz =
+// s + 8 j + out(j, k2) of rows k1 = s + 8 j < 2A, out[kx][iy][s][j][k2]; 16 lanes (J = 0):
+// kz = s + A k2 of row s < A, out[kx][iy][s][k2].  Entry = T[kx][iy][fold(kz)], fold(kz) =
+// min(kz, Mz - kz); rows past the last one are padding (zero).
+template <typename R>
+__global__ void k_vhat_lanes(const R* __restrict__ T, int rows, int hz, int Az, int J, int neg, R* __restrict__ out) {
+  const int Mz = 16 * Az, A2 = 2 * Az, fac = J ? 8 * J : 16, len = (J ? 8 : 16) * fac;
+  const size_t n = (size_t)rows * len;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t row = i / Mz;
-    const int p = (int)(i - row * Mz);
-    const int q = p / (4 * Az), rem = p - q * 4 * Az;
-    const int t = rem >> 2, k2 = 4 * q + (rem & 3);
-    const int kz = t + Az * k2;
-    out[i] = T[row * hz + (kz <= Mz / 2 ? kz : Mz - kz)];
-  }
-}
-
-// 8-lane order: entry p of a row is lane s = p / (2 Az), j = (p % (2 Az)) / 8, k2 = p % 8
-__global__ void k_vhat_lanes8(const float* __restrict__ T, int rows, int hz, int Az, float* __restrict__ out) {
-  const int Mz = 16 * Az, A2 = 2 * Az;
-  const size_t n = (size_t)rows * Mz;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t row = i / Mz;
-    const int p = (int)(i - row * Mz);
-    const int s = p / A2, rem = p - s * A2;
-    const int j = rem >> 3, k2 = rem & 7;
-    const int kz = (s + 8 * j) + A2 * k2;
-    out[i] = T[row * hz + (kz <= Mz / 2 ? kz : Mz - kz)];
+    const size_t row = i / len;
+    const int p = (int)(i - row * len);
+    const int s = p / fac, rem = p - s * fac;
+    const int j = J ? rem >> 3 : 0, k2 = J ? rem & 7 : rem, k1 = s + 8 * j;
+    R v = R(0);
+    if (k1 < (J ? A2 : Az)) {
+      const int kz = J ? k1 + A2 * (8 * j >= neg ? (k2 + 7) & 7 : k2) : k1 + Az * k2;
+      v = T[row * hz + (kz <= Mz / 2 ? kz : Mz - kz)];
+    }
+    out[i] = v;
   }
 }
 
 // ---------------------------------------------------------------------------------
 // host launchers
 
-cudaError_t launch_vhat_lanes8(const Geom& g, const float* table, float* out, cudaStream_t s) {
+template <typename R>
+cudaError_t launch_vhat_lanes(const Geom& g, const R* table, R* out, cudaStream_t s) {
   const int rows = (g.Mx / 2 + 1) * (g.My / 2 + 1);
-  k_vhat_lanes8<<<1024, 256, 0, s>>>(table, rows, g.Mz / 2 + 1, g.Az, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_vhat_lanes(const Geom& g, const float* table, float* out, cudaStream_t s) {
-  const int rows = (g.Mx / 2 + 1) * (g.My / 2 + 1);
-  k_vhat_lanes<<<1024, 256, 0, s>>>(table, rows, g.Mz / 2 + 1, g.Az, out);
+  const int J = p2_lanes<R>(g.Az) == 8 ? line_j(g.Az) : 0;
+  k_vhat_lanes<R><<<1024, 256, 0, s>>>(table, rows, g.Mz / 2 + 1, g.Az, J, line_neg(g.Az), out);
   return cudaGetLastError();
 }
 
@@ -860,6 +848,7 @@ cudaError_t launch_pair_products(const R* A, int na, const R* B, int nb, size_t 
 }
 
 #define RSX_INST(R)                                                                                        \
+  template cudaError_t launch_vhat_lanes<R>(const Geom&, const R*, R*, cudaStream_t);                     \
   template cudaError_t launch_gram<R>(const R*, int, const R*, int, size_t, double*, int, cudaStream_t,   \
                                       const R*, int*);                                                          \
   template cudaError_t launch_gram_reduce<R>(const double*, int, int, int, double, bool, double*, R*,      \

@@ -9,10 +9,9 @@ namespace rsx {
 cudaError_t launch_ghat(const Geom& g, double h, double scale, const double* cos_z, const double* cos_y,
                         const double* cos_x, double* buf0, double* buf1, void* table, bool fp64,
                         cudaStream_t s);
-// FP32 kernel table in pass 2's lane order, (Mx/2+1)(My/2+1) Mz floats (k_vhat_lanes)
-cudaError_t launch_vhat_lanes(const Geom& g, const float* table, float* out, cudaStream_t s);
-// the kernel table in the 8-lane y/z kernel's order [kx][|ky|][s][j][k2], kz = (s + 8 j) + 2 Az k2
-cudaError_t launch_vhat_lanes8(const Geom& g, const float* table, float* out, cudaStream_t s);
+// the kernel table in pass 2's lane order, (Mx/2+1)(My/2+1) rows of p2_row_factors<R>(Az) values (k_vhat_lanes)
+template <typename R>
+cudaError_t launch_vhat_lanes(const Geom& g, const R* table, R* out, cudaStream_t s);
 // part[blk][a][b] = partial sums of X_a(r) Y_b(r) w(r) (w may be null); na * nb <= 4096.
 // A kernel that gives up a bounded wait writes NaN partials and raises RSX_ETIMEOUT in *status.
 template <typename R>

@@ -434,6 +434,39 @@ RSX_HD void dft4_two_out(Cx<R>* v) {   // W: 1 -> {0, 1}, 3 -> {0, 3}, 12 -> {1,
   }
 }
 
+// 4-point DFT of which only the inputs A0 and A0 + 1 (mod 4) are non-zero: X_k = w^(A0 k)
+// (x_A0 + w^k x_(A0+1)), w = S i, four additions
+template <int S, int A0, typename R>
+RSX_HD void dft4_in_adjacent(Cx<R>& x0, Cx<R>& x1, Cx<R>& x2, Cx<R>& x3) {
+  const Cx<R> a = A0 == 0 ? x0 : A0 == 1 ? x1 : A0 == 2 ? x2 : x3;
+  const Cx<R> b = A0 == 0 ? x1 : A0 == 1 ? x2 : A0 == 2 ? x3 : x0;
+  const Cx<R> ia = mul_si<S>(a), ib = mul_si<S>(b);
+  x0 = a + b;
+  x2 = (A0 & 1) ? b - a : a - b;
+  if constexpr (A0 == 0) {
+    x1 = a + ib;
+    x3 = a - ib;
+  } else if constexpr (A0 == 1) {
+    x1 = ia - b;
+    x3 = cx<R>(-ia.x, -ia.y) - b;
+  } else if constexpr (A0 == 2) {
+    x1 = cx<R>(-a.x, -a.y) - ib;
+    x3 = ib - a;
+  } else {
+    x1 = b - ia;
+    x3 = b + ia;
+  }
+}
+// 4-point DFT, all inputs, forming only the outputs flagged true (in place)
+template <int S, bool W0, bool W1, bool W2, bool W3, typename R>
+RSX_HD void dft4_out(Cx<R>& x0, Cx<R>& x1, Cx<R>& x2, Cx<R>& x3) {
+  const Cx<R> a = x0 + x2, b = x0 - x2, c = x1 + x3, d = mul_si<S>(x1 - x3);
+  if constexpr (W0) x0 = a + c;
+  if constexpr (W2) x2 = a - c;
+  if constexpr (W1) x1 = b + d;
+  if constexpr (W3) x3 = b - d;
+}
+
 // 2-point DFTs with zero inputs skipped / unwanted outputs not formed (in place)
 template <bool N0, bool N1, typename R>
 RSX_HD void dft2_in(Cx<R>& x0, Cx<R>& x1) {
@@ -462,7 +495,7 @@ RSX_HD void dft2_out(Cx<R>& x0, Cx<R>& x1) {
   }
 }
 
-// Pruned Good-Thomas DFTs of length N = P Q (P = 2 or 3, gcd(P, Q) = 1), the index maps
+// Pruned Good-Thomas DFTs of length N = P Q (P = 2, 3 or 4, gcd(P, Q) = 1), the index maps
 // of DftPfa: input (Q n1 + P n2) mod N, output (Q qinv k1 + P pinv k2) mod N.
 //   half in  (inputs N/2 .. N zero): per column n2 the P-point DFT over n1 skips the zero
 //            inputs, then the Q-point DFTs over n2 are complete;
@@ -483,11 +516,16 @@ struct PfaHalfInCols {   // columns n2 = C .. Q-1
   RSX_HD static void run(const Cx<R>* v, Cx<R> (&y)[P][Q]) {
     if constexpr (C < Q) {
       using M = PfaMap<P, Q>;
-      constexpr bool m0 = M::in_nz(0, C), m1 = M::in_nz(1, C), m2 = M::in_nz(2, C);
+      constexpr bool m0 = M::in_nz(0, C), m1 = M::in_nz(1, C), m2 = M::in_nz(2, C), m3 = M::in_nz(3, C);
       if constexpr (m0) y[0][C] = v[M::in(0, C)];
       if constexpr (m1) y[1][C] = v[M::in(1, C)];
       if constexpr (P == 2) {
         dft2_in<m0, m1>(y[0][C], y[1][C]);
+      } else if constexpr (P == 4) {   // the four inputs are N/4 apart: exactly two adjacent ones are non-zero
+        static_assert(m0 + m1 + m2 + m3 == 2 && m0 != m2, "two adjacent inputs");
+        if constexpr (m2) y[2][C] = v[M::in(2, C)];
+        if constexpr (m3) y[3][C] = v[M::in(3, C)];
+        dft4_in_adjacent<S, (m0 && m1) ? 0 : (m1 && m2) ? 1 : (m2 && m3) ? 2 : 3>(y[0][C], y[1][C], y[2][C], y[3][C]);
       } else {
         if constexpr (m2) y[2][C] = v[M::in(2, C)];
         dft3_in<S, m0, m1, m2>(y[0][C], y[1][C], y[2][C]);
@@ -503,9 +541,12 @@ struct PfaHalfOutCols {   // columns k2 = C .. Q-1
   RSX_HD static void run(Cx<R> (&y)[P][Q], Cx<R>* out) {
     if constexpr (C < Q) {
       using M = PfaMap<P, Q>;
-      constexpr bool w0 = M::out_kept(0, C), w1 = M::out_kept(1, C), w2 = M::out_kept(2, C);
+      constexpr bool w0 = M::out_kept(0, C), w1 = M::out_kept(1, C), w2 = M::out_kept(2, C), w3 = M::out_kept(3, C);
       if constexpr (P == 2) {
         dft2_out<w0, w1>(y[0][C], y[1][C]);
+      } else if constexpr (P == 4) {
+        dft4_out<S, w0, w1, w2, w3>(y[0][C], y[1][C], y[2][C], y[3][C]);
+        if constexpr (w3) out[M::out(3, C)] = y[3][C];
       } else {
         if constexpr (w0 || w1 || w2) dft3_out<S, w0, w1, w2>(y[0][C], y[1][C], y[2][C]);
       }
@@ -551,12 +592,16 @@ template <int S> struct DftHalfIn<6, S> : DftPfaHalfIn<2, 3, S> {};
 template <int S> struct DftHalfIn<10, S> : DftPfaHalfIn<2, 5, S> {};
 template <int S> struct DftHalfIn<12, S> : DftPfaHalfIn<3, 4, S> {};
 template <int S> struct DftHalfIn<14, S> : DftPfaHalfIn<2, 7, S> {};
+template <int S> struct DftHalfIn<20, S> : DftPfaHalfIn<4, 5, S> {};
 template <int S> struct DftHalfIn<24, S> : DftPfaHalfIn<3, 8, S> {};
+template <int S> struct DftHalfIn<28, S> : DftPfaHalfIn<4, 7, S> {};
 template <int S> struct DftHalfOut<6, S> : DftPfaHalfOut<2, 3, S> {};
 template <int S> struct DftHalfOut<10, S> : DftPfaHalfOut<2, 5, S> {};
 template <int S> struct DftHalfOut<12, S> : DftPfaHalfOut<3, 4, S> {};
 template <int S> struct DftHalfOut<14, S> : DftPfaHalfOut<2, 7, S> {};
+template <int S> struct DftHalfOut<20, S> : DftPfaHalfOut<4, 5, S> {};
 template <int S> struct DftHalfOut<24, S> : DftPfaHalfOut<3, 8, S> {};
+template <int S> struct DftHalfOut<28, S> : DftPfaHalfOut<4, 7, S> {};
 
 // The 16-point DFT of which only outputs 0 .. 7 are wanted: Dft<16>'s radix-4 steps with
 // the second 4-point DFTs forming outputs k2 = 0, 1 only (k = k1 + 4 k2 < 8).

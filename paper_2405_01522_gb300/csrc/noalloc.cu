@@ -82,15 +82,13 @@ int exchange_noalloc(rsx_ctx* c, const void* phi, int nocc, const void* psi, int
   pm.nb = npsi;
   pm.N = N;
   Cx<R>* inter = (Cx<R>*)scratch;
-  const Cx<R>* twz = (const Cx<R>*)c->tw[0];
-  const Cx<R>* twy = (const Cx<R>*)c->tw[1];
   const Cx<R>* twx = (const Cx<R>*)c->tw[2];
   const int per_sm = std::max(1, pass2_occupancy<R>(g));
   const int grid = (int)std::min<long long>((long long)nocc * g.Hx, (long long)per_sm * c->nsm);
   for (int p = 0; p < npsi; ++p) {
     int rc = check_cuda(c, launch_pass1<R>(g, pm, p * nocc, nocc, inter, twx, s), "noalloc pass 1");
     if (rc) return rc;
-    rc = check_cuda(c, launch_pass2<R>(g, nocc, inter, twy, twz, (const R*)c->vhat, (const float*)c->vhatz, nullptr, grid, s),
+    rc = check_cuda(c, launch_pass2<R>(g, nocc, inter, (const Cx<R>*)c->twl, (const R*)c->vlanes, nullptr, grid, s),
                     "noalloc pass 2");
     if (rc) return rc;
     rc = check_cuda(c, launch_pass3<R>(g, pm, p * nocc, p, 1, 0, inter, twx, (R*)out + (size_t)p * N, s),

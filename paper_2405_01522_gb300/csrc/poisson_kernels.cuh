@@ -95,24 +95,6 @@ __device__ __forceinline__ void stage2_load(Cx<R> (&u)[16], int s, const Cx<R>* 
     for (int j = 0; j < 16; ++j) u[j] = sc[s * PITCH + j];
   }
 }
-// the transposed store: lane s writes its 16 values to scratch row s
-template <typename R, int PITCH = kScrPitch>
-__device__ __forceinline__ void stage2_store(const Cx<R> (&u)[16], int s, Cx<R>* sc) {
-  if constexpr (sizeof(R) == 4 && PITCH % 2 == 0) {
-    float4* rp = reinterpret_cast<float4*>(sc + s * PITCH);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) rp[j] = make_float4(u[2 * j].x, u[2 * j].y, u[2 * j + 1].x, u[2 * j + 1].y);
-  } else {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) sc[s * PITCH + j] = u[j];
-  }
-}
-
-// line-scratch pitch (complex) of pass 2: 18 for FP32 where the extra bytes fit (rows on
-// 16-byte boundaries for the vector loads above, still conflict-free), else 17
-template <typename R>
-__host__ __device__ constexpr int p2_pitch(int A) { return (sizeof(R) == 4 && A <= 12) ? 18 : kScrPitch; }
-
 // Row-block staging of the x passes, xs[kx][r] (kRowsPerCta = 32 rows per kx): the rows
 // are paired into 16 granules (r, r + 1 with r even) and granule g of row kx sits at
 // position g ^ (kx & 15), so that the 16 lanes of a line, which read granule `line` of 16
@@ -264,23 +246,10 @@ __global__ void __launch_bounds__(kThreads) k_pass1(Geom g, PairMap<R> pm, int q
 }
 
 // ---------------------------------------------------------------------------------
-// pass 2 pieces.  D is the (nz x My) plane of one (pair, kx), row pitch DP = My + 1.
-// Row loops step over pairs of rows per warp so that both half-warps of a warp run
-// the same number of iterations (their __syncwarp calls must match).
-
-template <int NT, typename R>
-__device__ __forceinline__ void load_plane(Cx<R>* D, int DP, const Cx<R>* P, int nz, int ny) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int z = warp; z < nz; z += NT / 32)
-    for (int y = lane; y < ny; y += 32) D[z * DP + y] = P[z * ny + y];
-}
-
-template <int NT, typename R>
-__device__ __forceinline__ void store_plane(const Cx<R>* D, int DP, Cx<R>* P, int nz, int ny) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int z = warp; z < nz; z += NT / 32)
-    for (int y = lane; y < ny; y += 32) P[z * ny + y] = D[z * DP + y];
-}
+// Pieces of the spectrum kernel.  D is the (nz x My) plane of one (pair, kx), row pitch
+// DP = My + 1.  Row loops step over pairs of rows per warp so that both half-warps of a warp
+// run the same number of iterations (their __syncwarp calls must match).  (Pass 2 itself is
+// in poisson_pass2.cuh.)
 
 // forward y transform of rows z < nz (input y < ny, output all My)
 template <typename R, int AY, int NT, int PITCH = kScrPitch>
@@ -317,69 +286,6 @@ __device__ __forceinline__ void y_forward(Cx<R>* D, int DP, int nz, int ny, cons
   }
 }
 
-// inverse y transform of rows z < nz (input all My of D's rows, output y < ny written to
-// out[z * opitch + y]: back into D, or straight to the plane in global memory)
-template <typename R, int AY, int NT, int PITCH = kScrPitch>
-__device__ __forceinline__ void y_inverse(Cx<R>* D, int DP, int nz, int ny, const Cx<R>* __restrict__ twy,
-                                          Cx<R>* sc, Cx<R>* out = nullptr, int opitch = 0) {
-  if (out == nullptr) {
-    out = D;
-    opitch = DP;
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 15;
-  // this lane's stage-1 twiddles (conjugated below), the same for every row
-  Cx<R> tw[AY];
-  if constexpr (AY % 2 == 0) {
-#pragma unroll
-    for (int k1 = 1; k1 < AY; ++k1) tw[k1] = twy[t * AY + k1];
-  }
-  for (int z0 = 2 * warp; z0 < nz; z0 += NT / 16) {
-    const int z = z0 + (lane >> 4);
-    const bool ok = z < nz;
-    Cx<R> v[AY];
-#pragma unroll
-    for (int a = 0; a < AY; ++a) v[a] = ok ? D[z * DP + t + 16 * a] : cx<R>(R(0), R(0));
-    if constexpr (AY % 2 == 0) {
-      Dft<AY, 1>::run(v);
-#pragma unroll
-      for (int k1 = 1; k1 < AY; ++k1) v[k1] = cmul(v[k1], conj(tw[k1]));
-#pragma unroll
-      for (int k1 = 0; k1 < AY; ++k1) sc[k1 * PITCH + t] = v[k1];
-    } else {
-      stage1_store<AY, 1, R, PITCH>(v, t, twy, sc);
-    }
-    __syncwarp();
-    Cx<R> u[16];
-    if (t < AY) {
-      stage2_load<R, PITCH>(u, t, sc);
-      if constexpr (AY % 2 == 0) {
-        Cx<R> o[8];
-        DftHalfOut<16, 1>::run(u, o);   // only y = t + AY k2 < ny = 8 AY, i.e. k2 < 8
-#pragma unroll
-        for (int k2 = 0; k2 < 8; ++k2) u[k2] = o[k2];
-      } else {
-        Dft<16, 1>::run(u);
-      }
-    }
-    __syncwarp();
-    if (ok && t < AY) {
-#pragma unroll
-      for (int k2 = 0; k2 < ((AY % 2 == 0) ? 8 : 16); ++k2) {
-        const int y = t + AY * k2;
-        if (y < ny) out[z * opitch + y] = u[k2];
-      }
-    }
-    __syncwarp();
-  }
-}
-
-// pass 2: per (pair, kx) plane: y forward, z forward * vhat * z inverse, y inverse.
-// pass2_plane is the body for one plane P (nz x ny, contiguous) at column kx; D is the
-// (nz x My) work plane (row pitch My + 1) and scr the line scratch.
-// Input staging: with `prefetched` the plane already sits in the upper half of the D rows
-// (columns [ny, 2 ny), copied by cp.async), otherwise it is loaded here into [0, ny).
-// With `Pnext` not null, the next plane is cp.async-prefetched into the upper halves
-// (dead after the y inverse) while this plane is stored.
 template <typename R>
 __device__ __forceinline__ void prefetch_plane_upper(Cx<R>* D, int DP, const Cx<R>* P, int nz, int ny, int NT) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -395,156 +301,6 @@ __device__ __forceinline__ void prefetch_plane_upper(Cx<R>* D, int DP, const Cx<
                      : "memory");
     }
   asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-template <typename R, int AY, int AZ, int NT>
-__device__ __forceinline__ void pass2_plane(const Geom& g, Cx<R>* P, int kx, const Cx<R>* __restrict__ twy,
-                                            const Cx<R>* __restrict__ twz, const R* __restrict__ vhat,
-                                            const float* __restrict__ vlanes, Cx<R>* D, Cx<R>* scr,
-                                            bool prefetched = false, const Cx<R>* Pnext = nullptr) {
-  constexpr int LY = 16 * AY;
-  constexpr int LZ = 16 * AZ;
-  constexpr int AMAX = AY > AZ ? AY : AZ;
-  constexpr int PITCH = p2_pitch<R>(AMAX);
-  constexpr int SP = AMAX * PITCH;
-  constexpr int DP = LY + 1;
-  constexpr int NZ = 8 * AZ, NY = 8 * AY;   // the box edges (the padded edge M = 16 A is 2n)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = lane & 15, line = warp * 2 + (lane >> 4);
-  Cx<R>* sc = scr + line * SP;
-  constexpr int Hy = LY / 2 + 1, Hz = LZ / 2 + 1;
-  if (prefetched) {
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-  } else {
-    load_plane<NT>(D, DP, P, NZ, NY);
-  }
-  __syncthreads();
-  y_forward<R, AY, NT, PITCH>(D, DP, NZ, NY, twy, sc, prefetched ? NY : 0);
-  __syncthreads();
-  // z forward, multiply, z inverse on columns ky (LY is a multiple of 16: uniform trips)
-  const R* vrow = vhat + (size_t)kx * Hy * Hz;
-  // this lane's forward stage-1 twiddles, the same for every column
-  Cx<R> twf[AZ];
-  if constexpr (AZ % 2 == 0) {
-#pragma unroll
-    for (int k1 = 1; k1 < AZ; ++k1) twf[k1] = twz[t * AZ + k1];
-  }
-  for (int ky = line; ky < LY; ky += NT / 16) {
-    const int iy = ky <= LY / 2 ? ky : LY - ky;
-    const R* vcol = vrow + (size_t)iy * Hz;
-    constexpr int AIN = (AZ % 2 == 0) ? AZ / 2 : AZ;   // inputs z >= nz = 8 AZ are zero
-    Cx<R> v[AZ];
-#pragma unroll
-    for (int a = 0; a < AIN; ++a) {
-      const int z = t + 16 * a;
-      v[a] = (z < NZ) ? D[z * DP + ky] : cx<R>(R(0), R(0));
-    }
-    if constexpr (AZ % 2 == 0) {
-      stage1_store_halfin_reg<AZ, R, PITCH>(v, t, twf, sc);
-    } else {
-      stage1_store<AZ, -1, R, PITCH>(v, t, twz, sc);
-    }
-    __syncwarp();
-    Cx<R> u[16];
-    if (t < AZ) stage2_load<R, PITCH>(u, t, sc);
-    __syncwarp();
-    if (t < AZ) {
-      Dft<16, -1>::run(u);
-      if constexpr (sizeof(R) == 4) {
-        // four 16-byte loads per lane from the lane-order table (k_vhat_lanes): the
-        // factors of kz = t + AZ k2, k2 = 4 j .. 4 j + 3
-        const float4* vq = reinterpret_cast<const float4*>(vlanes + ((size_t)kx * Hy + iy) * LZ) + t;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 m = __ldg(vq + j * AZ);
-          u[4 * j] = cscale(u[4 * j], m.x);
-          u[4 * j + 1] = cscale(u[4 * j + 1], m.y);
-          u[4 * j + 2] = cscale(u[4 * j + 2], m.z);
-          u[4 * j + 3] = cscale(u[4 * j + 3], m.w);
-        }
-      } else {
-#pragma unroll
-        for (int k2 = 0; k2 < 16; ++k2) {
-          const int kz = t + AZ * k2;
-          const R m = __ldg(vcol + (kz <= LZ / 2 ? kz : LZ - kz));
-          u[k2] = cx<R>(u[k2].x * m, u[k2].y * m);
-        }
-      }
-      Dft<16, 1>::run(u);
-      if constexpr (AZ % 2 == 0) {
-        stage2_store<R, PITCH>(u, t, sc);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          Cx<R> w = twz[j * AZ + t];
-          w.y = -w.y;
-          sc[t * PITCH + j] = cmul(u[j], w);
-        }
-      }
-    }
-    __syncwarp();
-    Cx<R> r[AZ];
-#pragma unroll
-    for (int k1 = 0; k1 < AZ; ++k1) r[k1] = sc[k1 * PITCH + t];
-    if constexpr (AZ % 2 == 0) {
-      // the inverse twiddle w_M^{-j k1} (j the 16-point output index) taken after the
-      // transpose, where lane t = j holds k1 = 0 .. AZ-1: the conjugates of the forward
-      // twiddles this lane already holds, instead of 16 table loads per column
-#pragma unroll
-      for (int k1 = 1; k1 < AZ; ++k1) r[k1] = cmul(r[k1], conj(twf[k1]));
-      Cx<R> o[AZ / 2];
-      DftHalfOut<AZ, 1>::run(r, o);   // only z = t + 16 a < nz = 8 AZ, i.e. a < AZ / 2
-#pragma unroll
-      for (int a = 0; a < AZ / 2; ++a) D[(t + 16 * a) * DP + ky] = o[a];
-    } else {
-      Dft<AZ, 1>::run(r);
-#pragma unroll
-      for (int a = 0; a < AZ; ++a) {
-        const int z = t + 16 * a;
-        if (z < NZ) D[z * DP + ky] = r[a];
-      }
-    }
-    __syncwarp();
-  }
-  __syncthreads();
-  // the inverse rows go straight to the plane in global memory (no copy through D)
-  y_inverse<R, AY, NT, PITCH>(D, DP, NZ, NY, twy, sc, P, NY);
-  __syncthreads();   // every read of D's upper halves is done
-  if (Pnext) prefetch_plane_upper<R>(D, DP, Pnext, NZ, NY, NT);
-}
-
-// D lives in shared memory (DSMEM) or, when it does not fit, in a per-CTA slice of
-// global scratch.  Persistent grid over the work items (pair, kx).
-template <typename R, int AY, int AZ, bool DSMEM, int NT>
-__global__ void __launch_bounds__(NT, 1) k_pass2(Geom g, int nq, Cx<R>* __restrict__ inter,
-                                                 const Cx<R>* __restrict__ twy, const Cx<R>* __restrict__ twz,
-                                                 const R* __restrict__ vhat, const float* __restrict__ vlanes,
-                                                 R* gscratch) {
-  constexpr int AMAX = AY > AZ ? AY : AZ;
-  constexpr int SP = AMAX * p2_pitch<R>(AMAX);
-  constexpr int DP = 16 * AY + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Cx<R>* scr = reinterpret_cast<Cx<R>*>(smem_raw);
-  Cx<R>* D = DSMEM ? scr + (NT / 16) * SP
-                   : reinterpret_cast<Cx<R>*>(gscratch) + (size_t)blockIdx.x * g.nz * DP;
-  const int nplane = g.nz * g.ny;
-  const int nwork = nq * g.Hx;
-  auto plane_ptr = [&](int w) {
-    const int ql = w / g.Hx, kx = w - ql * g.Hx;
-    return inter + (size_t)ql * g.inter_elems() + (size_t)kx * nplane;
-  };
-  // in shared memory the next plane is prefetched behind the current one (2 ny <= My + 1)
-  const bool pipe = DSMEM;
-  if (pipe && (int)blockIdx.x < nwork) prefetch_plane_upper<R>(D, DP, plane_ptr(blockIdx.x), 8 * AZ, 8 * AY, NT);
-  for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
-    if (!RSX_IN_RANGE(g, (long long)(w / g.Hx) * g.inter_elems() + (long long)(w % g.Hx + 1) * nplane - 1,
-                      (long long)nq * g.inter_elems()))
-      break;   // whole CTA: its work index decides
-    const int kx = w % g.Hx;
-    const int wn = w + (int)gridDim.x;
-    pass2_plane<R, AY, AZ, NT>(g, plane_ptr(w), kx, twy, twz, vhat, vlanes, D, scr, pipe,
-                               (pipe && wn < nwork) ? plane_ptr(wn) : nullptr);
-  }
 }
 
 // Casida pair spectra (panel tile-major, see below): per (transition q, kx) plane, y forward and z forward, then

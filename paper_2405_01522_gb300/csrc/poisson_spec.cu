@@ -32,10 +32,10 @@ cudaError_t launch_spectrum_f32(const Geom& g, int nq, const Cx<float>* inter, c
   // memory.  (Dividing n evenly with fewer lines, e.g. 320 threads at n = 80, measured
   // slower than 512 with one partial round.)
   int nt = spectrum_threads(g.Ay);
-  size_t smem = pass2_scratch_smem<float>(g.Ay, g.Az, nt) + pass2_plane_bytes<float>(g);
+  size_t smem = spectrum_smem(g, nt);
   if (smem > (size_t)max_dyn_smem()) {
     nt = 256;
-    smem = pass2_scratch_smem<float>(g.Ay, g.Az, nt) + pass2_plane_bytes<float>(g);
+    smem = spectrum_smem(g, nt);
   }
   if (smem > (size_t)max_dyn_smem()) return cudaErrorInvalidValue;
   int dev = 0, nsm = 0;

@@ -88,12 +88,9 @@ struct Geom {
   int Mz, My, Mx;     // padded (2n)
   int Az, Ay, Ax;     // M / 16
   int Hx;             // Mx / 2 + 1 (half spectrum along x)
-  int p2_threads;     // tuning: threads per CTA of the y/z pass (256 or 512)
   int p1_group;       // tuning: pass-1 block order (0: pair-major; G > 0: pairs fastest in groups of G)
   int p2_global;      // tuning: 1 = the y/z pass keeps its work plane in global scratch even where
                       // shared memory would hold it (0 = shared memory whenever it fits)
-  int p2_lanes;       // tuning: lanes per line of the y/z transforms, 16 (16 x A) or 8 (8 x 2A;
-                      // FP32, A a multiple of 4, shared-memory plane)
   int* dbg = nullptr; // bounds-checked builds: the status word an out-of-range index is reported in
   int dbg_nq = 0;     // bounds-checked builds: pairs the launch's intermediate holds (0: unknown)
   __host__ __device__ size_t N() const { return (size_t)nz * ny * nx; }
@@ -119,14 +116,11 @@ __device__ inline bool in_range_checked(int* dbg, long long i, long long n) {
 template <typename R>
 cudaError_t launch_pass1(const Geom& g, const PairMap<R>& pm, int q0, int nq, Cx<R>* inter,
                          const Cx<R>* twx, cudaStream_t s);
-// tw8 / vl8: twiddles and lane-order kernel table of the 8-lane split (FP32; NULL: the
-// 16-lane kernel runs whatever g.p2_lanes says)
+// twl: w_M^{-t k1}, t < lanes, k1 < M / lanes (lanes per line: 8, or 16 in FP32 at edge 112);
+// vlanes: the kernel table in the y/z pass's lane order (launch_vhat_lanes)
 template <typename R>
-cudaError_t launch_pass2(const Geom& g, int nq, Cx<R>* inter, const Cx<R>* twy, const Cx<R>* twz,
-                         const R* vhat, const float* vhat_lanes, R* gscratch, int grid, cudaStream_t s,
-                         const Cx<float>* tw8 = nullptr, const float* vl8 = nullptr);
-// true when the 8-lane y/z kernel serves geometry g (FP32) with these tables
-bool pass2_l8_active(const Geom& g, const void* tw8, const void* vl8);
+cudaError_t launch_pass2(const Geom& g, int nq, Cx<R>* inter, const Cx<R>* twl, const R* vlanes, R* gscratch, int grid,
+                         cudaStream_t s);
 template <typename R>
 cudaError_t launch_pass3(const Geom& g, const PairMap<R>& pm, int q0, int p0, int np, int pot, const Cx<R>* inter,
                          const Cx<R>* twx, R* out, cudaStream_t s);
@@ -139,6 +133,8 @@ cudaError_t launch_spectrum_f32(const Geom& g, int nq, const Cx<float>* inter, c
 cudaError_t launch_spectrum_weights(const Geom& g, const float* vhat, float h3, float* wsq, cudaStream_t s);
 template <typename R>
 size_t pass2_smem_bytes(const Geom& g, bool* fits);
+template <typename R>
+size_t pass2_gscratch_bytes(const Geom& g, int grid);   // global plane scratch of a launch of `grid` CTAs
 template <typename R>
 int pass2_occupancy(const Geom& g);  // resident pass-2 CTAs per SM (shared-memory variant)
 

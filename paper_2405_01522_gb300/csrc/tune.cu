@@ -1,25 +1,19 @@
 // Autotuner for the pair-solve path.
 //
-// Knobs (rsx_tuning, per box size, precision and device):
-//   - p2_threads: threads per CTA of the y/z pass, 256, 384 (FP32) or 512, each used only
-//     where its line scratch and the work plane fit in shared memory;
-//   - p2_global: the y/z pass keeps its (nz x My) work plane in shared memory (one CTA per
-//     SM, next plane prefetched behind the current one) or in a global scratch slice per
-//     CTA that stays in L2 (only the line scratch in shared memory);
-//   - p2_lanes: the radix split of the y/z line transforms (M = 16 A points), 16 lanes x A
-//     or 8 lanes x 2A (FP32, A in {4, 8, 12});
+// Knobs searched (rsx_tuning, per box size, precision and device):
 //   - p1_group: the x pass's block order, pair-major (0) or pairs fastest in groups of G
 //     (CTAs in flight share their orbital rows in L2);
 //   - chunk_outputs: output orbitals per exchange chunk, 1, 2, 4 or all (small chunks keep
 //     a chunk's pair intermediates near L2 size between the passes, large chunks launch
 //     fewer, fuller grids).
-// The search is coordinate descent from the current knobs: the pass-2 configuration
-// (threads x plane staging x line split) first, then the pass-1 order, then the chunking, each
-// candidate timed on the exchange apply of synthetic orbitals on the device (one warm-up,
-// best of two runs, CUDA events).  The winner is applied to the context and appended to
-// a text cache keyed by (edges, precision, nocc, npsi, SMs, device name), so later
-// contexts skip the timing.  Only p2_lanes changes the arithmetic (the rounding order of
-// the line transforms); under the other knobs the results are bitwise the same.
+// The y/z pass has one kernel per edge and precision (poisson_pass2.cuh), so p2_threads and
+// p2_lanes choose nothing; p2_global (the work plane in global scratch) stays as the caller
+// set it: it measured three times slower wherever shared memory holds the plane.
+// The search is coordinate descent from the current knobs, each candidate timed on the
+// exchange apply of synthetic orbitals on the device (one warm-up, best of two runs, CUDA
+// events).  The winner is applied to the context and appended to a text cache keyed by
+// (edges, precision, nocc, npsi, SMs, device name), so later contexts skip the timing.  The
+// results are bitwise the same under every knob.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -91,21 +85,21 @@ bool valid(const rsx_tuning& t) {
 }
 
 void apply(rsx_ctx* c, const rsx_tuning& t) {
-  c->g.p2_threads = t.p2_threads;
+  c->p2_threads = t.p2_threads;
+  c->p2_lanes = t.p2_lanes;
   c->g.p1_group = t.p1_group;
   c->g.p2_global = t.p2_global;
-  c->g.p2_lanes = t.p2_lanes;
   c->p2_occ[0] = c->p2_occ[1] = 0;
   c->chunk_outputs = t.chunk_outputs;
 }
 
 rsx_tuning current(const rsx_ctx* c) {
   rsx_tuning t;
-  t.p2_threads = c->g.p2_threads;
+  t.p2_threads = c->p2_threads;
   t.chunk_outputs = c->chunk_outputs;
   t.p1_group = c->g.p1_group;
   t.p2_global = c->g.p2_global;
-  t.p2_lanes = c->g.p2_lanes;
+  t.p2_lanes = c->p2_lanes;
   return t;
 }
 
@@ -197,32 +191,14 @@ extern "C" int rsx_autotune_ex(rsx_ctx* c, int nocc, int npsi, const char* cache
         best = t;
       }
     };
-    // 1. pass-2 configuration: CTA size x plane staging x line split
-    const int p2s[3] = {256, 384, 512};
-    const bool l8 = c->precision == RSX_FP32 && pass2_l8_active(
-        [&] { Geom g8 = c->g; g8.p2_lanes = 8; g8.p2_global = 0; return g8; }(), c->tw8, c->vhatz8);
-    for (int a = 0; a < 3; ++a) {
-      if (a > 0 && c->precision != RSX_FP32) break;
-      for (int gl = 0; gl < 2; ++gl) {
-        if (gl == 1 && a > 0) continue;   // the global-plane kernel runs at 256 threads
-        for (int ln = 0; ln < 2; ++ln) {
-          if (ln == 1 && (!l8 || gl == 1 || a == 2)) continue;   // 8 lanes: shared plane, 256 or 384 threads
-          rsx_tuning t = best;
-          t.p2_threads = p2s[a];
-          t.p2_global = gl;
-          t.p2_lanes = ln ? 8 : 16;
-          consider(t);
-        }
-      }
-    }
-    // 2. pass-1 block order
+    // 1. pass-1 block order
     const int groups[5] = {0, 4, 16, 64, 1 << 30};
     for (int gi = 0; gi < 5; ++gi) {
       rsx_tuning t = best;
       t.p1_group = groups[gi];
       consider(t);
     }
-    // 3. output orbitals per chunk
+    // 2. output orbitals per chunk
     const int chs[4] = {1, 2, 4, 0};
     for (int b = 0; b < 4; ++b) {
       if (chs[b] >= npsi) continue;
