@@ -112,6 +112,22 @@ namespace {
 
 bool edge_ok(int n) { return n >= 16 && n % 8 == 0 && axis_supported(n / 8); }
 
+// table [k1][t] of w_M^{-t k1}, t < lanes, k1 < M / lanes, on the device
+template <typename R>
+cudaError_t line_twiddles(rsx_ctx* c, int M, int lanes, void** out) {
+  const int rad = M / lanes;
+  std::vector<Cx<R>> tw(M);
+  for (int t = 0; t < lanes; ++t)
+    for (int k1 = 0; k1 < rad; ++k1) {
+      const double ang = 2.0 * M_PI * (double)(t * k1) / (double)M;
+      tw[k1 * lanes + t].x = (R)cos(ang);
+      tw[k1 * lanes + t].y = (R)(-sin(ang));
+    }
+  size_t have = 0;
+  if (grow(c, out, &have, tw.size() * sizeof(Cx<R>), "line twiddles") != RSX_OK) return cudaErrorMemoryAllocation;
+  return cudaMemcpy(*out, tw.data(), tw.size() * sizeof(Cx<R>), cudaMemcpyHostToDevice);
+}
+
 template <typename R>
 int make_tables(rsx_ctx* c) {
   const Geom& g = c->g;
@@ -155,21 +171,12 @@ int make_tables(rsx_ctx* c) {
   const double scale = c->h * c->h * c->h / npad;
   cudaError_t e = launch_ghat(g, c->h, scale, dcos[0], dcos[1], dcos[2], b0, b1, c->vhat, sizeof(R) == 8, 0);
   if (e == cudaSuccess) {
-    // the y/z pass: its lane-order table and twiddles w_M^{-t k1}, t < lanes, k1 < M / lanes
-    size_t have_vl = 0, have_tw = 0;
-    const int lanes = p2_lanes<R>(g.Az), rad = g.Mz / lanes;
-    std::vector<Cx<R>> twl(g.Mz);
-    for (int t = 0; t < lanes; ++t)
-      for (int k1 = 0; k1 < rad; ++k1) {
-        const double ang = 2.0 * M_PI * (double)(t * k1) / (double)g.Mz;
-        twl[t * rad + k1].x = (R)cos(ang);
-        twl[t * rad + k1].y = (R)(-sin(ang));
-      }
-    if (grow(c, &c->vlanes, &have_vl, (size_t)hx * hy * p2_row_factors<R>(g.Az) * sizeof(R), "kernel table (lane order)") != RSX_OK ||
-        grow(c, &c->twl, &have_tw, twl.size() * sizeof(Cx<R>), "line twiddles") != RSX_OK)
+    // the y/z pass's lane-order table; the line twiddles w_M^{-t k1}, t < lanes, k1 < M / lanes
+    size_t have_vl = 0;
+    if (grow(c, &c->vlanes, &have_vl, (size_t)hx * hy * p2_row_factors<R>(g.Az) * sizeof(R), "kernel table (lane order)") != RSX_OK)
       e = cudaErrorMemoryAllocation;
-    else
-      e = cudaMemcpy(c->twl, twl.data(), twl.size() * sizeof(Cx<R>), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = line_twiddles<R>(c, g.Mz, p2_lanes<R>(g.Az), &c->twl);
+    if (e == cudaSuccess) e = line_twiddles<R>(c, g.Mx, 8, &c->twx);
     if (e == cudaSuccess) e = launch_vhat_lanes<R>(g, (const R*)c->vhat, (R*)c->vlanes, 0);
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -212,7 +219,7 @@ int solve_pairs(rsx_ctx* c, const PairMap<R>& pm, int q0, int nq, int p0, int np
   int rc = grow(c, &c->work, &c->work_bytes, need, "FFT intermediates");
   if (rc) return rc;
   Cx<R>* inter = (Cx<R>*)c->work;
-  const Cx<R>* twx = (const Cx<R>*)c->tw[2];
+  const Cx<R>* twx = (const Cx<R>*)c->twx;
   {
     ProfScope ps(c, kKPass1, s);
     rc = check_cuda(c, launch_pass1<R>(g, pm, q0, nq, inter, twx, s), "pass 1");
@@ -461,7 +468,7 @@ int rsx_destroy(rsx_ctx* c) {
   cudaDeviceSynchronize();
   prof_collect(c);
   for (cudaEvent_t e : c->prof_pool) cudaEventDestroy(e);
-  void* bufs[] = {c->vhat, c->vlanes, c->twl, c->tw[0], c->tw[1], c->tw[2], c->work, c->gscr, c->dsm, c->smallr, c->status,
+  void* bufs[] = {c->vhat, c->vlanes, c->twl, c->twx, c->tw[0], c->tw[1], c->tw[2], c->work, c->gscr, c->dsm, c->smallr, c->status,
                   c->panel_hi, c->panel_lo, c->gemm_part, c->eig_work, c->gscr_kd, c->pos, c->tdhf_work, c->specw, c->ones};
   for (void* b : bufs)
     if (b) cudaFree(b);

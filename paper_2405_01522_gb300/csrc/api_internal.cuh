@@ -29,6 +29,7 @@ struct rsx_ctx {
   void* vhat = nullptr;                 // kernel table T[kx][ky][kz] (R)
   void* vlanes = nullptr;               // the same in pass 2's lane order (R, launch_vhat_lanes)
   void* twl = nullptr;                  // y/z line twiddles w_M^{-t k1}, t < lanes, k1 < M / lanes (R)
+  void* twx = nullptr;                  // x line twiddles w_M^{-t k1}, t < 8, k1 < 2 Ax (R)
   void* tw[3] = {nullptr, nullptr, nullptr};
   void* work = nullptr;   size_t work_bytes = 0;     // FFT intermediates
   void* gscr = nullptr;   size_t gscr_bytes = 0;     // pass-2 planes when shared memory is too small

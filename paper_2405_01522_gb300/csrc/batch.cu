@@ -122,7 +122,7 @@ int record(rsx_batch* b, cudaStream_t s) {
     pm.N = c->g.N();
     pm.plist = grp.plist;
     pm.olist = grp.olist;
-    const Cx<float>* twx = (const Cx<float>*)c->tw[2];
+    const Cx<float>* twx = (const Cx<float>*)c->twx;
     rc = bcuda(b, launch_pass1<float>(c->g, pm, 0, grp.npairs, inter, twx, s), "batch pass 1");
     if (rc) return rc;
     const long long nwork = (long long)grp.npairs * c->g.Hx;

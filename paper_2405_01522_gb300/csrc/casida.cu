@@ -151,7 +151,7 @@ int casida_K_f32(rsx_ctx* c, const TSet* sets, int nsets, double* K, cudaStream_
       if (!sets[k].nt()) continue;
       const PairMap<float> pm = prod_map<float>(sets[k].pv, sets[k].nv, sets[k].po, sets[k].no, N);  // q = i * nv + a
       rc = check_cuda(c, launch_pass1<float>(g, pm, 0, sets[k].nt(), inter + off * g.inter_elems(),
-                                             (const Cx<float>*)c->tw[2], s),
+                                             (const Cx<float>*)c->twx, s),
                       "pass 1");
       off += sets[k].nt();
     }

@@ -494,20 +494,24 @@ __global__ void k_pair_products(const R* __restrict__ A, int na, const R* __rest
   }
 }
 
-// Pass 2's copy of the kernel table in the order its lanes read it (poisson_lines.cuh), as
-// consecutive values per lane and folded column (kx, |ky|).  8 lanes: lane s holds kz =
-// s + 8 j + out(j, k2) of rows k1 = s + 8 j < 2A, out[kx][iy][s][j][k2]; 16 lanes (J = 0):
-// kz = s + A k2 of row s < A, out[kx][iy][s][k2].  Entry = T[kx][iy][fold(kz)], fold(kz) =
-// min(kz, Mz - kz); rows past the last one are padding (zero).
+// Pass 2's copy of the kernel table in the order its lanes read it (poisson_lines.cuh).  Lane
+// s uses fac values per folded column (kx, |ky|), number f the factor of
+//   8 lanes: kz = s + 8 j + out(j, k2), f = 8 j + k2 (rows k1 = s + 8 j < 2A),
+//   16 lanes (J = 0): kz = s + A f (s < A, f < 16),
+// in 16-byte pieces of E values, the lanes' pieces adjacent: out[kx][iy][f / E][s][f % E].
+// Entry = T[kx][iy][fold(kz)], fold(kz) = min(kz, Mz - kz); rows past the last one are padding
+// (zero).  (Each lane's values contiguous instead put the eight lanes of a 16-byte load on
+// eight lines: 32 L1 wavefronts per load, a sixth of the pass's.)
 template <typename R>
 __global__ void k_vhat_lanes(const R* __restrict__ T, int rows, int hz, int Az, int J, int neg, R* __restrict__ out) {
-  const int Mz = 16 * Az, A2 = 2 * Az, fac = J ? 8 * J : 16, len = (J ? 8 : 16) * fac;
+  constexpr int E = 16 / (int)sizeof(R);
+  const int Mz = 16 * Az, A2 = 2 * Az, lanes = J ? 8 : 16, fac = J ? 8 * J : 16, len = lanes * fac;
   const size_t n = (size_t)rows * len;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const size_t row = i / len;
     const int p = (int)(i - row * len);
-    const int s = p / fac, rem = p - s * fac;
-    const int j = J ? rem >> 3 : 0, k2 = J ? rem & 7 : rem, k1 = s + 8 * j;
+    const int s = (p / E) % lanes, f = p / (E * lanes) * E + p % E;
+    const int j = J ? f >> 3 : 0, k2 = J ? f & 7 : f, k1 = s + 8 * j;
     R v = R(0);
     if (k1 < (J ? A2 : Az)) {
       const int kz = J ? k1 + A2 * (8 * j >= neg ? (k2 + 7) & 7 : k2) : k1 + Az * k2;

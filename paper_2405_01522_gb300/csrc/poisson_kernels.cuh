@@ -95,156 +95,6 @@ __device__ __forceinline__ void stage2_load(Cx<R> (&u)[16], int s, const Cx<R>* 
     for (int j = 0; j < 16; ++j) u[j] = sc[s * PITCH + j];
   }
 }
-// Row-block staging of the x passes, xs[kx][r] (kRowsPerCta = 32 rows per kx): the rows
-// are paired into 16 granules (r, r + 1 with r even) and granule g of row kx sits at
-// position g ^ (kx & 15), so that the 16 lanes of a line, which read granule `line` of 16
-// different kx, hit distinct banks, and granules move with single 16-byte (FP32) accesses.
-__device__ __forceinline__ int xs_idx(int kx, int r) {
-  return kx * kRowsPerCta + ((((r >> 1) ^ (kx & 15))) << 1) + (r & 1);
-}
-
-// two consecutive complex values (one granule) from / to shared memory
-template <typename R>
-__device__ __forceinline__ void ld_granule(const Cx<R>* p, Cx<R>& a, Cx<R>& b) {
-  if constexpr (sizeof(R) == 4) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    a = cx<R>(v.x, v.y);
-    b = cx<R>(v.z, v.w);
-  } else {
-    a = p[0];
-    b = p[1];
-  }
-}
-template <typename R>
-__device__ __forceinline__ void st_granule(Cx<R>* p, Cx<R> a, Cx<R> b) {
-  if constexpr (sizeof(R) == 4) {
-    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
-  } else {
-    p[0] = a;
-    p[1] = b;
-  }
-}
-
-// ---------------------------------------------------------------------------------
-// pass 1: x forward (r2c via row pairs).  One item = (pair q, plane z, 32 rows).
-// pass1_item is the body (all threads of the CTA call it with the same item); the
-// intermediate of the pair is at `dst_pair` (layout [kx][z][y]).
-template <typename R, int AX>
-__device__ __forceinline__ void pass1_item(const Geom& g, const R* f1, const R* f2, int z, int yblk,
-                                           Cx<R>* __restrict__ dst_pair, const Cx<R>* __restrict__ twx,
-                                           unsigned char* smem_raw) {
-  constexpr int L = 16 * AX;
-  constexpr int SP = AX * kScrPitch;
-  constexpr int H = L / 2 + 1;
-  Cx<R>* scr = reinterpret_cast<Cx<R>*>(smem_raw);
-  Cx<R>* xs = scr;   // [H][kRowsPerCta], see xs_idx: reuses the line scratch once all lines are done with it
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = lane & 15, line = warp * 2 + (lane >> 4);
-  const int y0 = yblk * kRowsPerCta;
-  const int ya = y0 + 2 * line, yb = ya + 1;
-  Cx<R>* sc = scr + line * SP;
-  const size_t plane = (size_t)z * g.ny * g.nx;
-  f1 += plane;
-  f2 += plane;
-
-  constexpr int AIN = (AX % 2 == 0) ? AX / 2 : AX;   // inputs x >= nx = 8 AX are zero
-  Cx<R> v[AX];
-#pragma unroll
-  for (int a = 0; a < AIN; ++a) {
-    const int x = t + 16 * a;
-    R re = R(0), im = R(0);
-    if (x < g.nx) {
-      if (ya < g.ny && RSX_IN_RANGE(g, plane + (size_t)ya * g.nx + x, g.N()))
-        re = __ldg(f1 + (size_t)ya * g.nx + x) * __ldg(f2 + (size_t)ya * g.nx + x);
-      if (yb < g.ny && RSX_IN_RANGE(g, plane + (size_t)yb * g.nx + x, g.N()))
-        im = __ldg(f1 + (size_t)yb * g.nx + x) * __ldg(f2 + (size_t)yb * g.nx + x);
-    }
-    v[a] = cx<R>(re, im);
-  }
-  if constexpr (AX % 2 == 0) {
-    stage1_store_halfin<AX, -1>(v, t, twx, sc);
-  } else {
-    stage1_store<AX, -1>(v, t, twx, sc);
-  }
-  __syncwarp();
-  Cx<R> u[16];
-  if (t < AX) {
-    stage2_load(u, t, sc);
-    Dft<16, -1>::run(u);
-  }
-  __syncwarp();
-  if (t < AX) {
-#pragma unroll
-    for (int k2 = 0; k2 < 16; ++k2) sc[t + AX * k2] = u[k2];  // natural order U[k]
-  }
-  __syncwarp();
-  // split the packed line: X_a(k) = (U(k) + conj U(L-k)) / 2,  X_b(k) = (U(k) - conj U(L-k)) / 2i,
-  // into registers first: the staging buffer overwrites every line's scratch
-  constexpr int NK = (H + 15) / 16;
-  Cx<R> xa[NK], xb[NK];
-#pragma unroll
-  for (int i = 0; i < NK; ++i) {
-    const int k = t + 16 * i;
-    if (k < H) {
-      const Cx<R> U = sc[k];
-      const Cx<R> Um = sc[(L - k) % L];
-      xa[i] = cx<R>(R(0.5) * (U.x + Um.x), R(0.5) * (U.y - Um.y));
-      xb[i] = cx<R>(R(0.5) * (U.y + Um.y), R(-0.5) * (U.x - Um.x));
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NK; ++i) {
-    const int k = t + 16 * i;
-    if (k < H) st_granule(xs + xs_idx(k, 2 * line), xa[i], xb[i]);
-  }
-  __syncthreads();
-  const int nrow = min(kRowsPerCta, g.ny - y0);   // a multiple of 8 (ny = 8 A)
-  Cx<R>* dst = dst_pair + (size_t)z * g.ny + y0;
-  const size_t kstride = (size_t)g.nz * g.ny;
-  for (int e = threadIdx.x; e < H * (kRowsPerCta / 2); e += kThreads) {
-    const int kx = e / (kRowsPerCta / 2), r = 2 * (e - kx * (kRowsPerCta / 2));
-    if (r < nrow && RSX_IN_RANGE(g, (size_t)z * g.ny + y0 + (size_t)kx * kstride + r + 1, g.inter_elems())) {
-      Cx<R> a, b;
-      ld_granule(xs + xs_idx(kx, r), a, b);
-      st_granule(dst + (size_t)kx * kstride + r, a, b);
-    }
-  }
-  __syncthreads();
-}
-
-// Block order: with g.p1_group == 0 a pair's (z, row block) items are consecutive (long
-// contiguous runs of stores per kx); with g.p1_group = G > 0 the pairs are the fastest
-// index in groups of G, so that the CTAs in flight share (z, row block) and the orbital
-// rows they multiply are read from HBM once per group and then hit in L2.
-template <typename R, int AX>
-__global__ void __launch_bounds__(kThreads) k_pass1(Geom g, PairMap<R> pm, int q0, int nq, Cx<R>* __restrict__ inter,
-                                                    const Cx<R>* __restrict__ twx) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int nyb = (g.ny + kRowsPerCta - 1) / kRowsPerCta;
-  int b = blockIdx.x;
-  int yblk, z, ql;
-  if (g.p1_group <= 0) {
-    yblk = b % nyb;
-    b /= nyb;
-    z = b % g.nz;
-    ql = b / g.nz;  // local pair slot
-  } else {
-    const int lo = b % g.p1_group;
-    b /= g.p1_group;
-    yblk = b % nyb;
-    b /= nyb;
-    z = b % g.nz;
-    ql = (b / g.nz) * g.p1_group + lo;
-    if (ql >= nq) return;   // whole CTA: the last group is partial
-  }
-  if (!RSX_IN_RANGE(g, ql, nq)) return;   // whole CTA
-  const R* f1;
-  const R* f2;
-  pm.pair(q0 + ql, f1, f2);
-  pass1_item<R, AX>(g, f1, f2, z, yblk, inter + (size_t)ql * g.inter_elems(), twx, smem_raw);
-}
-
 // ---------------------------------------------------------------------------------
 // Pieces of the spectrum kernel.  D is the (nz x My) plane of one (pair, kx), row pitch
 // DP = My + 1.  Row loops step over pairs of rows per warp so that both half-warps of a warp
@@ -426,214 +276,6 @@ __global__ void __launch_bounds__(NT) k_spectrum(Geom g, int nq, const Cx<float>
       }
     }
   }
-}
-
-// ---------------------------------------------------------------------------------
-// pass 3: x inverse (c2r via row pairs) of every pair in output p's list, and
-// out_p(z, y, x) = - sum_e partner_e(z, y, x) V_e(z, y, x).  One item = (p, z, 32 rows).
-// With pot != 0 the output p is the potential V of pair q = p itself (no partner, no sign).
-// The next pair's row block and partner tile are copied with cp.async into the second
-// of two shared-memory buffers while the current pair is transformed.
-// pass3_item is the body; `out_p` is output p's array, `inter` the slot base of q0.
-
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// shared-memory bytes of pass 3 for element type R (two buffers of row block + tile)
-template <typename R>
-__host__ __device__ inline size_t pass3_buffer_elems(int AX, int nx) {
-  const int H = 8 * AX + 1;
-  return (size_t)H * kRowsPerCta * sizeof(Cx<R>) + (size_t)kRowsPerCta * nx * sizeof(R);
-}
-
-template <typename R, int AX>
-__device__ __forceinline__ void pass3_prefetch(const Geom& g, const PairMap<R>& pm, int q0, int p, int e, int z,
-                                               int y0, int nrow, int pot, const Cx<R>* __restrict__ inter,
-                                               Cx<R>* xs, R* tile) {
-  constexpr int H = 8 * AX + 1;
-  int q = p;
-  const R* partner = nullptr;
-  if (!pot) pm.entry(p, e, q, partner);
-  const Cx<R>* src = inter + (size_t)(q - q0) * g.inter_elems() + (size_t)z * g.ny + y0;
-  const size_t kstride = (size_t)g.nz * g.ny;
-  const bool slot_ok = RSX_IN_RANGE(g, q - q0, g.dbg_nq > 0 ? g.dbg_nq : 0x7fffffff);
-  // one granule (rows r, r + 1) per copy; the intermediate is library-owned and 16-byte
-  // aligned, nrow is a multiple of 8
-  for (int i = threadIdx.x; i < H * (kRowsPerCta / 2); i += kThreads) {
-    const int kx = i / (kRowsPerCta / 2), r = 2 * (i - kx * (kRowsPerCta / 2));
-    Cx<R>* dp = xs + xs_idx(kx, r);
-    if (r < nrow && slot_ok &&
-        RSX_IN_RANGE(g, (size_t)z * g.ny + y0 + (size_t)kx * kstride + r + 1, g.inter_elems())) {
-      const Cx<R>* sp = src + (size_t)kx * kstride + r;
-      cp_async16(dp, sp);
-      if (sizeof(R) == 8) cp_async16(dp + 1, sp + 1);
-    } else {
-      st_granule(dp, cx<R>(R(0), R(0)), cx<R>(R(0), R(0)));
-    }
-  }
-  if (!pot) {
-    const R* prow = partner + (size_t)z * g.ny * g.nx + (size_t)y0 * g.nx;
-    const int cnt = RSX_IN_RANGE(g, (size_t)z * g.ny * g.nx + (size_t)(y0 + nrow) * g.nx - 1, g.N()) ? nrow * g.nx : 0;
-    if (((reinterpret_cast<uintptr_t>(prow) | (uintptr_t)(cnt * sizeof(R))) & 15u) == 0) {
-      constexpr int V = 16 / (int)sizeof(R);
-      for (int i = threadIdx.x * V; i < cnt; i += kThreads * V) cp_async16(tile + i, prow + i);
-    } else {
-      for (int i = threadIdx.x; i < cnt; i += kThreads) {
-        if (sizeof(R) == 4)
-          cp_async4(tile + i, prow + i);
-        else
-          cp_async8(tile + i, prow + i);
-      }
-    }
-  }
-}
-
-template <typename R, int AX>
-__device__ __forceinline__ void pass3_item(const Geom& g, const PairMap<R>& pm, int q0, int p, int z, int yblk,
-                                           int pot, const Cx<R>* __restrict__ inter, const Cx<R>* __restrict__ twx,
-                                           R* __restrict__ out_p, unsigned char* smem_raw) {
-  constexpr int L = 16 * AX;
-  constexpr int SP = AX * kScrPitch;
-  constexpr int H = L / 2 + 1;
-  Cx<R>* scr = reinterpret_cast<Cx<R>*>(smem_raw);
-  unsigned char* buf0 = reinterpret_cast<unsigned char*>(scr + kLinesPerCta * SP);
-  const size_t bufbytes = pass3_buffer_elems<R>(AX, g.nx);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = lane & 15, line = warp * 2 + (lane >> 4);
-  const int y0 = yblk * kRowsPerCta;
-  const int nrow = min(kRowsPerCta, g.ny - y0);
-  Cx<R>* sc = scr + line * SP;
-  const size_t plane = (size_t)z * g.ny * g.nx;
-  auto xs_of = [&](int b) { return reinterpret_cast<Cx<R>*>(buf0 + b * bufbytes); };
-  auto tile_of = [&](int b) { return reinterpret_cast<R*>(buf0 + b * bufbytes + (size_t)H * kRowsPerCta * sizeof(Cx<R>)); };
-
-  R acc0[16], acc1[16];
-#pragma unroll
-  for (int k2 = 0; k2 < 16; ++k2) acc0[k2] = acc1[k2] = R(0);
-
-  // this lane's stage-1 twiddles, the same for every entry
-  Cx<R> tw[AX];
-  if constexpr (AX % 2 == 0) {
-#pragma unroll
-    for (int k1 = 1; k1 < AX; ++k1) tw[k1] = twx[t * AX + k1];
-  }
-  const int ne = pot ? 1 : pm.nentries(p);
-  __syncthreads();   // the buffers may still be read by a previous item of this CTA
-  pass3_prefetch<R, AX>(g, pm, q0, p, 0, z, y0, nrow, pot, inter, xs_of(0), tile_of(0));
-  cp_async_commit();
-  for (int e = 0; e < ne; ++e) {
-    if (e + 1 < ne) {
-      pass3_prefetch<R, AX>(g, pm, q0, p, e + 1, z, y0, nrow, pot, inter, xs_of((e + 1) & 1), tile_of((e + 1) & 1));
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const Cx<R>* xs = xs_of(e & 1);
-    const R* tile = tile_of(e & 1);
-
-    // Z(k) = X_a(k) + i X_b(k), Hermitian extension for k > L/2
-    Cx<R> v[AX];
-#pragma unroll
-    for (int a = 0; a < AX; ++a) {
-      const int k = t + 16 * a;
-      Cx<R> xa, xb;
-      if (k < H) {
-        ld_granule(xs + xs_idx(k, 2 * line), xa, xb);
-      } else {
-        ld_granule(xs + xs_idx(L - k, 2 * line), xa, xb);
-        xa = conj(xa);
-        xb = conj(xb);
-      }
-      v[a] = cx<R>(xa.x - xb.y, xa.y + xb.x);
-    }
-    if constexpr (AX % 2 == 0) {
-      Dft<AX, 1>::run(v);
-#pragma unroll
-      for (int k1 = 1; k1 < AX; ++k1) v[k1] = cmul(v[k1], conj(tw[k1]));
-#pragma unroll
-      for (int k1 = 0; k1 < AX; ++k1) sc[k1 * kScrPitch + t] = v[k1];
-    } else {
-      stage1_store<AX, 1>(v, t, twx, sc);
-    }
-    __syncwarp();
-    if (t < AX) {
-      Cx<R> u[16];
-      stage2_load(u, t, sc);
-      if constexpr (AX % 2 == 0) {
-        Cx<R> o[8];
-        DftHalfOut<16, 1>::run(u, o);   // only x = t + AX k2 < nx = 8 AX, i.e. k2 < 8
-#pragma unroll
-        for (int k2 = 0; k2 < 8; ++k2) u[k2] = o[k2];
-      } else {
-        Dft<16, 1>::run(u);
-      }
-      const int ra = 2 * line, rb = ra + 1;
-#pragma unroll
-      for (int k2 = 0; k2 < ((AX % 2 == 0) ? 8 : 16); ++k2) {
-        const int x = t + AX * k2;
-        if (x < g.nx) {
-          if (pot) {
-            acc0[k2] += u[k2].x;
-            acc1[k2] += u[k2].y;
-          } else {
-            if (ra < nrow) acc0[k2] -= tile[ra * g.nx + x] * u[k2].x;
-            if (rb < nrow) acc1[k2] -= tile[rb * g.nx + x] * u[k2].y;
-          }
-        }
-      }
-    }
-    __syncwarp();
-    __syncthreads();   // buffer e & 1 is refilled by the prefetch of entry e + 2
-  }
-  R* tile = tile_of(0);
-  if (t < AX) {
-    const int ra = 2 * line, rb = ra + 1;
-#pragma unroll
-    for (int k2 = 0; k2 < ((AX % 2 == 0) ? 8 : 16); ++k2) {   // x = t + AX k2 < nx = 8 AX
-      const int x = t + AX * k2;
-      if (x < g.nx) {
-        if (ra < nrow) tile[ra * g.nx + x] = acc0[k2];
-        if (rb < nrow) tile[rb * g.nx + x] = acc1[k2];
-      }
-    }
-  }
-  __syncthreads();
-  R* orow = out_p + plane + (size_t)y0 * g.nx;
-  if (RSX_IN_RANGE(g, plane + (size_t)(y0 + nrow) * g.nx - 1, g.N()))
-    for (int i = threadIdx.x; i < nrow * g.nx; i += kThreads) orow[i] = tile[i];
-  __syncthreads();
-}
-
-template <typename R, int AX>
-__global__ void __launch_bounds__(kThreads) k_pass3(Geom g, PairMap<R> pm, int q0, int p0, int pot,
-                                                    const Cx<R>* __restrict__ inter,
-                                                    const Cx<R>* __restrict__ twx, R* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  // outputs are the fastest index: the CTAs in flight share (z, row block), so the partner
-  // rows they multiply come from HBM once and then from L2 for the other outputs
-  const int nyb = (g.ny + kRowsPerCta - 1) / kRowsPerCta;
-  const int np = (int)(gridDim.x / ((unsigned)g.nz * nyb));
-  int b = blockIdx.x;
-  const int pl = b % np;
-  b /= np;
-  const int yblk = b % nyb;
-  const int z = b / nyb;
-  pass3_item<R, AX>(g, pm, q0, p0 + pl, z, yblk, pot, inter, twx, pm.out_row(p0 + pl, out, pl), smem_raw);
 }
 
 }  // namespace rsx

@@ -16,17 +16,6 @@ inline bool axis_supported_impl(int A) {
   }
 }
 
-// line scratch and the row-block staging buffer share the same bytes (pass1_item)
-template <typename R>
-inline size_t pass1_smem(int AX) {
-  const int L = 16 * AX, H = L / 2 + 1;
-  const size_t scr = (size_t)kLinesPerCta * AX * kScrPitch, xs = (size_t)H * kRowsPerCta;
-  return sizeof(Cx<R>) * (scr > xs ? scr : xs);
-}
-template <typename R>
-inline size_t pass3_smem(int AX, int nx) {
-  return sizeof(Cx<R>) * (size_t)kLinesPerCta * AX * kScrPitch + 2 * pass3_buffer_elems<R>(AX, nx);
-}
 inline int max_dyn_smem() {
   int dev = 0, v = 0;
   cudaGetDevice(&dev);

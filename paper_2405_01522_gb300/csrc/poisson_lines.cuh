@@ -34,22 +34,35 @@ struct Line {
   __host__ __device__ static constexpr int out(int j, int k2) { return A2 * (8 * j >= NEG ? (k2 + 7) & 7 : k2); }
 };
 
-// Scratch rows of 8 complex.  FP32 (64 bytes): row k1 of line l sits at physical row
-// k1 ^ (l & 1) and the four 16-byte chunks of physical row r are XOR-swizzled by
-// (r >> 1) & 3.  Then (i) the two lines of a half-warp put the same row in opposite halves
-// of the banks, so the 8-byte accesses of stage 1 are conflict-free, and (ii) the eight
-// lanes of a line reading rows s + 8 j as 16-byte chunks hit eight distinct bank groups.
-// FP64 (128 bytes): element t of row r sits at t ^ (r & 7): conflict-free both ways.
-template <typename R>
+// Scratch rows of 8 complex, element t of row r of line l at off(r, t, l) (l: the line's number
+// in its warp, lines' scratch a multiple of 128 bytes apart).  Two lane orders of a warp's
+// four lines:
+//   t fastest (lane 8 l + t; the y/z pass).  FP32: the row sits at r ^ (l & 1) and its four
+//     16-byte chunks are XOR-swizzled by (row >> 1) & 3.  Then (i) the two lines of a half-warp
+//     put the same row in opposite halves of the banks, so the 8-byte accesses of stage 1 are
+//     conflict-free, and (ii) the eight lanes of a line reading rows s + 8 j as 16-byte
+//     chunks hit eight distinct bank groups.  FP64 (128-byte rows): element t at t ^ (r & 7).
+//   l fastest (lane 4 t + l; the x passes, whose 16-byte global accesses coalesce over the four
+//     lines only if these are consecutive lanes).  FP32: the row sits at r ^ l, its chunks are
+//     swizzled by row bit 1 (as 2) and row bit 2 (as 1) and by l & 1: 4 lines x 4 lanes of a
+//     half-warp cover the banks once in stage 1, and so do 4 lines x 2 rows of a quarter-warp
+//     in stage 2.  FP64: element t at t ^ (r & 7) ^ 2 l.
+template <typename R, bool LFAST>
 struct LineScr;
 
-template <>
-struct LineScr<float> {
-  static __device__ __forceinline__ int par(int line) { return line & 1; }
-  static __device__ __forceinline__ int off(int r, int t) { return r * 8 + 2 * ((t >> 1) ^ ((r >> 1) & 3)) + (t & 1); }
-  static __device__ __forceinline__ void load(Cx<float> (&u)[8], const Cx<float>* sc, int r) {
-    const int sw = (r >> 1) & 3;
-    const float4* rp = reinterpret_cast<const float4*>(sc + r * 8);
+template <bool LFAST>
+struct LineScr<float, LFAST> {
+  static __device__ __forceinline__ int row(int r, int l) { return LFAST ? r ^ l : r ^ (l & 1); }
+  static __device__ __forceinline__ int swz(int pr, int l) {
+    return LFAST ? ((pr & 2) | ((pr >> 2) & 1)) ^ (l & 1) : (pr >> 1) & 3;
+  }
+  static __device__ __forceinline__ int off(int r, int t, int l) {
+    const int pr = row(r, l);
+    return pr * 8 + 2 * ((t >> 1) ^ swz(pr, l)) + (t & 1);
+  }
+  static __device__ __forceinline__ void load(Cx<float> (&u)[8], const Cx<float>* sc, int r, int l) {
+    const int pr = row(r, l), sw = swz(pr, l);
+    const float4* rp = reinterpret_cast<const float4*>(sc + pr * 8);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float4 v = rp[q ^ sw];
@@ -57,47 +70,46 @@ struct LineScr<float> {
       u[2 * q + 1] = cx<float>(v.z, v.w);
     }
   }
-  static __device__ __forceinline__ void store(Cx<float>* sc, int r, const Cx<float> (&u)[8]) {
-    const int sw = (r >> 1) & 3;
-    float4* rp = reinterpret_cast<float4*>(sc + r * 8);
+  static __device__ __forceinline__ void store(Cx<float>* sc, int r, int l, const Cx<float> (&u)[8]) {
+    const int pr = row(r, l), sw = swz(pr, l);
+    float4* rp = reinterpret_cast<float4*>(sc + pr * 8);
 #pragma unroll
     for (int q = 0; q < 4; ++q) rp[q ^ sw] = make_float4(u[2 * q].x, u[2 * q].y, u[2 * q + 1].x, u[2 * q + 1].y);
   }
 };
 
-template <>
-struct LineScr<double> {
-  static __device__ __forceinline__ int par(int) { return 0; }
-  static __device__ __forceinline__ int off(int r, int t) { return r * 8 + (t ^ (r & 7)); }
-  static __device__ __forceinline__ void load(Cx<double> (&u)[8], const Cx<double>* sc, int r) {
+template <bool LFAST>
+struct LineScr<double, LFAST> {
+  static __device__ __forceinline__ int off(int r, int t, int l) { return r * 8 + (t ^ (r & 7) ^ (LFAST ? 2 * l : 0)); }
+  static __device__ __forceinline__ void load(Cx<double> (&u)[8], const Cx<double>* sc, int r, int l) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const double2 v = *reinterpret_cast<const double2*>(sc + off(r, q));
+      const double2 v = *reinterpret_cast<const double2*>(sc + off(r, q, l));
       u[q] = cx<double>(v.x, v.y);
     }
   }
-  static __device__ __forceinline__ void store(Cx<double>* sc, int r, const Cx<double> (&u)[8]) {
+  static __device__ __forceinline__ void store(Cx<double>* sc, int r, int l, const Cx<double> (&u)[8]) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) *reinterpret_cast<double2*>(sc + off(r, q)) = make_double2(u[q].x, u[q].y);
+    for (int q = 0; q < 8; ++q) *reinterpret_cast<double2*>(sc + off(r, q, l)) = make_double2(u[q].x, u[q].y);
   }
 };
 
 // This lane's twiddles w_M^{-t k}, k <= W, in registers, or (REG = false) read from the
-// table tw8[t][k1] where they are used.
+// table tw8[k1][t] where they are used.
 template <typename R, int A, bool REG = true>
 struct LineTw {
   Cx<R> reg[REG ? Line<A>::W + 1 : 1];
   const Cx<R>* tab;
   __device__ __forceinline__ void init(const Cx<R>* __restrict__ tw8, int t) {
-    tab = tw8 + t * Line<A>::A2;
+    tab = tw8 + t;
     if constexpr (REG) {
 #pragma unroll
-      for (int k = 1; k <= Line<A>::W; ++k) reg[k] = tab[k];
+      for (int k = 1; k <= Line<A>::W; ++k) reg[k] = tab[8 * k];
     }
   }
   __device__ __forceinline__ Cx<R> get(int k) const {
     if constexpr (REG) return reg[k];
-    else return tab[k];
+    else return tab[8 * k];
   }
   // row k1 times w^{-t k1} (forward) or w^{+t k1} (inverse), k1 >= 1
   __device__ __forceinline__ Cx<R> fwd(Cx<R> x, int k1) const {
@@ -110,21 +122,21 @@ struct LineTw {
 
 // The 8-lane split as used by a kernel: JP groups of 8 rows pass through the line's scratch at
 // a time (JP = J: all at once), TWREG: twiddles in registers.
-__host__ __device__ constexpr int line_rows(int A, int jp) { return jp >= line_j(A) ? 2 * A : 8 * jp; }
+__host__ __device__ constexpr int line_rows(int A, int jp) { return jp >= line_j(A) ? (2 * A + 3) / 4 * 4 : 8 * jp; }
 
-template <typename R, int A, int JP, bool TWREG = true>
+template <typename R, int A, int JP, bool TWREG = true, bool LFAST = false>
 struct Split8 {
   using L = Line<A>;
+  using Scr = LineScr<R, LFAST>;
   using Tw = LineTw<R, A, TWREG>;
   static constexpr int LANES = 8, NIN = A, RAD = 8, FAC = 8 * L::J, SCR = line_rows(A, JP) * 8;
-  static __device__ __forceinline__ int par(int line) { return LineScr<R>::par(line); }
   __host__ __device__ static constexpr int out(int j, int k2) { return L::out(j, k2); }
 
-  // Forward line: v[a] is input t + 8 a < n = 8 A; `put(k, x)` receives X[k] (lane t: the 8-point
-  // spectra of rows k1 = t + 8 j).
-  template <class Put>
-  static __device__ __forceinline__ void forward(const Cx<R> (&v)[A], int t, int par, unsigned lmask, const Tw& tw,
-                                                 Cx<R>* sc, Put put) {
+  // Forward line: v[a] is input t + 8 a < n = 8 A; `row(j, k1, u)` receives the 8-point spectra
+  // u[k2] = X[k1 + out(j, k2)] of this lane's rows k1 = t + 8 j.
+  template <class Row>
+  static __device__ __forceinline__ void forward_rows(const Cx<R> (&v)[A], int t, int l, unsigned lmask, const Tw& tw,
+                                                      Cx<R>* sc, Row row) {
     Cx<R> x[L::A2];
     DftHalfIn<L::A2, -1>::run(v, x);
 #pragma unroll
@@ -132,26 +144,36 @@ struct Split8 {
 #pragma unroll
     for (int p = 0; p < L::J; p += JP) {
 #pragma unroll
-      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) sc[LineScr<R>::off((k1 - 8 * p) ^ par, t)] = x[k1];
+      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) sc[Scr::off(k1 - 8 * p, t, l)] = x[k1];
       __syncwarp(lmask);
 #pragma unroll
       for (int j = p; j < p + JP && j < L::J; ++j) {
         const int k1 = t + 8 * j;
         if (8 * j + 8 <= L::A2 || k1 < L::A2) {
           Cx<R> u[8];
-          LineScr<R>::load(u, sc, (k1 - 8 * p) ^ par);
+          Scr::load(u, sc, k1 - 8 * p, l);
           Dft<8, -1>::run(u);
-#pragma unroll
-          for (int k2 = 0; k2 < 8; ++k2) put(k1 + out(j, k2), u[k2]);
+          row(j, k1, u);
         }
       }
       __syncwarp(lmask);
     }
   }
+  // the same with `put(k, x)` receiving X[k]
+  template <class Put>
+  static __device__ __forceinline__ void forward(const Cx<R> (&v)[A], int t, int l, unsigned lmask, const Tw& tw,
+                                                 Cx<R>* sc, Put put) {
+    forward_rows(v, t, l, lmask, tw, sc, [&](int j, int k1, const Cx<R>(&u)[8]) {
+#pragma unroll
+      for (int k2 = 0; k2 < 8; ++k2) put(k1 + out(j, k2), u[k2]);
+    });
+  }
 
-  // Inverse line: `in(k)` gives X[k]; `put(i, x)` receives output i < n.
-  template <class In, class Put>
-  static __device__ __forceinline__ void inverse(int t, int par, unsigned lmask, const Tw& tw, Cx<R>* sc, In in, Put put) {
+  // Inverse line: `row(j, k1, u)` fills u[k2] with X[k1 + out(j, k2)] of row k1 = t + 8 j;
+  // `put(a, i, x)` receives output i = t + 8 a < n.
+  template <class Row, class Put>
+  static __device__ __forceinline__ void inverse_rows(int t, int l, unsigned lmask, const Tw& tw, Cx<R>* sc, Row row,
+                                                      Put put) {
     Cx<R> r[L::A2], o[A];
 #pragma unroll
     for (int p = 0; p < L::J; p += JP) {
@@ -160,28 +182,57 @@ struct Split8 {
         const int k1 = t + 8 * j;
         if (8 * j + 8 <= L::A2 || k1 < L::A2) {
           Cx<R> u[8];
-#pragma unroll
-          for (int k2 = 0; k2 < 8; ++k2) u[k2] = in(k1 + out(j, k2));
+          row(j, k1, u);
           Dft<8, 1>::run(u);
-          LineScr<R>::store(sc, (k1 - 8 * p) ^ par, u);
+          Scr::store(sc, k1 - 8 * p, l, u);
         }
       }
       __syncwarp(lmask);
 #pragma unroll
-      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) r[k1] = sc[LineScr<R>::off((k1 - 8 * p) ^ par, t)];
+      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) r[k1] = sc[Scr::off(k1 - 8 * p, t, l)];
       __syncwarp(lmask);
     }
 #pragma unroll
     for (int k1 = 1; k1 < L::A2; ++k1) r[k1] = tw.inv(r[k1], k1);
     DftHalfOut<L::A2, 1>::run(r, o);
 #pragma unroll
-    for (int a = 0; a < A; ++a) put(t + 8 * a, o[a]);
+    for (int a = 0; a < A; ++a) put(a, t + 8 * a, o[a]);
   }
+  // the same with `in(k)` giving X[k] and `put(i, x)`
+  template <class In, class Put>
+  static __device__ __forceinline__ void inverse(int t, int l, unsigned lmask, const Tw& tw, Cx<R>* sc, In in, Put put) {
+    inverse_rows(
+        t, l, lmask, tw, sc,
+        [&](int j, int k1, Cx<R>(&u)[8]) {
+#pragma unroll
+          for (int k2 = 0; k2 < 8; ++k2) u[k2] = in(k1 + out(j, k2));
+        },
+        [&](int, int i, Cx<R> x) { put(i, x); });
+  }
+
+  // Two real rows packed as one complex line have their half spectra in U(k) and U(M - k).  Lane
+  // t holds X at (row j, k2): k = t + 8 j + 2A k2; M - k is in lane (2A - t) mod 8 at
+  //   row JF - j (lanes t <= 2A mod 8), row JF - 1 - j (the others), JF = floor(2A / 8), and 7 - k2;
+  // k1 = 0 (lane 0, row 0) pairs with itself at (8 - k2) mod 8.  mirror(j, k2, get) returns the
+  // partner lane's get(row, 7 - k2) for this lane's (j, k2): get reads this lane's own values at
+  // compile-time rows.  Valid rows only; lane 0 row 0 takes its own value instead.
+  static constexpr int JF = L::A2 / 8, RM = L::A2 % 8;
+  template <class Get>
+  static __device__ __forceinline__ Cx<R> mirror(int j, int k2, int t, Get get) {
+    static_assert(LFAST, "lane order of the x passes");
+    const int ja = JF - j < L::J ? JF - j : L::J - 1, jb = JF - 1 - j >= 0 ? JF - 1 - j : 0;
+    const Cx<R> va = get(ja, 7 - k2), vb = get(jb, 7 - k2);
+    const bool ca = t <= RM;
+    const int src = (((RM - t) & 7) << 2) | (threadIdx.x & 3);   // lanes 4 t + l
+    return cx<R>(__shfl_sync(0xffffffffu, ca ? va.x : vb.x, src), __shfl_sync(0xffffffffu, ca ? va.y : vb.y, src));
+  }
+  // register index of logical k2 in row j (negative rows are rotated by one)
+  __host__ __device__ static constexpr int reg(int j, int k2) { return 8 * j >= L::NEG ? (k2 + 1) & 7 : k2; }
 
   // Forward, multiply by the factors, inverse: the spectrum stays in registers and scratch
   // rows; `scale(j, u)` multiplies the 8 spectra of row t + 8 j.
   template <class In, class Scale, class Put>
-  static __device__ __forceinline__ void convolve(int t, int par, unsigned lmask, const Tw& tw, Cx<R>* sc, In in,
+  static __device__ __forceinline__ void convolve(int t, int l, unsigned lmask, const Tw& tw, Cx<R>* sc, In in,
                                                   Scale scale, Put put) {
     Cx<R> v[A], x[L::A2], o[A];
 #pragma unroll
@@ -192,23 +243,23 @@ struct Split8 {
 #pragma unroll
     for (int p = 0; p < L::J; p += JP) {
 #pragma unroll
-      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) sc[LineScr<R>::off((k1 - 8 * p) ^ par, t)] = x[k1];
+      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) sc[Scr::off(k1 - 8 * p, t, l)] = x[k1];
       __syncwarp(lmask);
 #pragma unroll
       for (int j = p; j < p + JP && j < L::J; ++j) {
         const int k1 = t + 8 * j;
         if (8 * j + 8 <= L::A2 || k1 < L::A2) {
           Cx<R> u[8];
-          LineScr<R>::load(u, sc, (k1 - 8 * p) ^ par);
+          Scr::load(u, sc, k1 - 8 * p, l);
           Dft<8, -1>::run(u);
           scale(j, u);
           Dft<8, 1>::run(u);
-          LineScr<R>::store(sc, (k1 - 8 * p) ^ par, u);   // read and written by this lane only
+          Scr::store(sc, k1 - 8 * p, l, u);   // read and written by this lane only
         }
       }
       __syncwarp(lmask);
 #pragma unroll
-      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) x[k1] = sc[LineScr<R>::off((k1 - 8 * p) ^ par, t)];
+      for (int k1 = 8 * p; k1 < 8 * (p + JP) && k1 < L::A2; ++k1) x[k1] = sc[Scr::off(k1 - 8 * p, t, l)];
       __syncwarp(lmask);
     }
 #pragma unroll
@@ -229,12 +280,11 @@ struct Split16 {
   using R = float;
   static_assert(A % 2 == 0, "even A");
   static constexpr int LANES = 16, NIN = A / 2, RAD = 16, FAC = 16, PITCH = 17, SCR = A * PITCH;
-  static __device__ __forceinline__ int par(int) { return 0; }
   struct Tw {
     Cx<R> reg[A];
     __device__ __forceinline__ void init(const Cx<R>* __restrict__ tw, int t) {
 #pragma unroll
-      for (int k = 1; k < A; ++k) reg[k] = tw[t * A + k];
+      for (int k = 1; k < A; ++k) reg[k] = tw[16 * k + t];
     }
   };
   static __device__ __forceinline__ void stage1(const Cx<R> (&v)[NIN], int t, const Tw& tw, Cx<R>* sc) {

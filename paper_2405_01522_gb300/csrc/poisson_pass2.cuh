@@ -71,8 +71,9 @@ __device__ __forceinline__ void p2_scale4(Cx<float>* u, float4 m) {
 // registers, inverts the row it holds, and writes the new spectrum over it.  (With the next
 // plane staged through shared memory behind the y inverse, its load was exposed once per
 // plane and a plane took four barriers instead of two.)
-// tw[t][k1] = w_M^{-t k1} (t < 8, k1 < 2A; 16 lanes: t < 16, k1 < A); vl: the kernel table in
-// the split's lane order, FAC values per lane and folded column (k_vhat_lanes).
+// tw[k1][t] = w_M^{-t k1} (t < 8, k1 < 2A; 16 lanes: t < 16, k1 < A); vl: the kernel table in
+// the split's lane order, FAC values per lane and folded column, the lanes' 16-byte pieces
+// adjacent (k_vhat_lanes).
 // Shared memory: [line scratch] [plane NB x p2_pitch].
 template <typename R, int A, bool DSMEM>
 __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cx<R>* scr = reinterpret_cast<Cx<R>*>(smem_raw);
   Cx<R>* D = DSMEM ? scr + NL * S::SCR : gscratch + (size_t)blockIdx.x * NB * DP;
-  const int lane = threadIdx.x & 31, t = lane & (LN - 1), line = threadIdx.x / LN, par = S::par(line);
+  const int lane = threadIdx.x & 31, t = lane & (LN - 1), line = threadIdx.x / LN, l = line & 3;
   const unsigned lmask = (LN == 8 ? 0xFFu : 0xFFFFu) << (lane & (32 - LN));
   // the two lines of a half-warp (line 2k, 2k + 1) take rows 4 apart and columns 1 apart, see
   // p2_pitch (the last four lines of an odd half block of 8 keep their own rows)
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
   };
   auto y_forward = [&](int z) {   // outputs all M columns
     Cx<R>* row = D + z * DP;
-    S::forward(v, t, par, lmask, tw, sc, [&](int k, Cx<R> x) { row[k] = x; });
+    S::forward(v, t, l, lmask, tw, sc, [&](int k, Cx<R> x) { row[k] = x; });
   };
   Cx<R>* P = plane_ptr(blockIdx.x);
   if (P) {
@@ -129,7 +130,8 @@ __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
     // ---- z forward, kernel multiply, z inverse on the M columns ky.  Columns ky and M - ky
     // use the same kernel factors (the table is folded in |ky|): a line takes them as one
     // item (item 0: the two unpaired columns 0 and M / 2) and loads the factors once.
-    const R* vrow = vl + (size_t)kx * Hy * FROW + t * S::FAC;
+    constexpr int E = 16 / (int)sizeof(R);   // values per 16-byte piece
+    const R* vrow = vl + (size_t)kx * Hy * FROW + t * E;
     for (int it = line; it < M / 2; it += NL) {
       float4 fac[S::FAC / 4];
 #pragma unroll 1
@@ -139,12 +141,12 @@ __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
         if constexpr (sizeof(R) == 4) {
           if (c == 0 || it == 0) {
 #pragma unroll
-            for (int i = 0; i < S::FAC / 4; ++i) fac[i] = __ldg(reinterpret_cast<const float4*>(vsrc) + i);
+            for (int i = 0; i < S::FAC / 4; ++i) fac[i] = __ldg(reinterpret_cast<const float4*>(vsrc) + i * LN);
           }
         }
         Cx<R>* col = D + ky;
         S::convolve(
-            t, par, lmask, tw, sc, [&](int i) { return col[i * DP]; },
+            t, l, lmask, tw, sc, [&](int i) { return col[i * DP]; },
             [&](int j, Cx<R>(&u)[S::RAD]) {
               if constexpr (sizeof(R) == 4) {
 #pragma unroll
@@ -152,7 +154,7 @@ __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
               } else {
 #pragma unroll
                 for (int k2 = 0; k2 < S::RAD; k2 += 2) {
-                  const double2 m = __ldg(reinterpret_cast<const double2*>(vsrc + S::RAD * j + k2));
+                  const double2 m = __ldg(reinterpret_cast<const double2*>(vsrc) + (S::RAD * j + k2) / 2 * LN);
                   u[k2] = cscale(u[k2], m.x);
                   u[k2 + 1] = cscale(u[k2 + 1], m.y);
                 }
@@ -168,7 +170,7 @@ __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
       if (kAhead && Pn) load_row(Pn, z);
       const Cx<R>* row = D + z * DP;
       Cx<R>* dst = P + (size_t)z * NB;
-      S::inverse(t, par, lmask, tw, sc, [&](int k) { return row[k]; }, [&](int i, Cx<R> x) { dst[i] = x; });
+      S::inverse(t, l, lmask, tw, sc, [&](int k) { return row[k]; }, [&](int i, Cx<R> x) { dst[i] = x; });
       if (Pn) {
         if (!kAhead) load_row(Pn, z);
         y_forward(z);

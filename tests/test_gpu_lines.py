@@ -32,3 +32,32 @@ def test_yz_pass_at_every_edge(edge, prec, nocc, npsi):
     assert torch.equal(a, b)
     ref = oracle.exchange_apply(s.phi, s.psi, h)
     assert rel_max_err(a.double().cpu().numpy(), ref) < TOL[prec]
+
+
+def _off(x, k):
+    """A contiguous copy of x starting k elements into its buffer (off 16-byte boundaries)."""
+    buf = torch.empty(x.numel() + k, dtype=x.dtype, device=x.device)
+    buf[k:] = x.reshape(-1)
+    return buf[k:].view(x.shape)
+
+
+@pytest.mark.parametrize("prec,nx", [("fp32", 24), ("fp32", 40), ("fp32", 112), ("fp64", 24), ("fp64", 56)])
+def test_x_passes_off_sixteen_byte_boundaries(prec, nx):
+    """Orbitals and outputs that start off 16-byte boundaries take the element-wise row copies
+    of the x passes: the same bits as the aligned call, for x edges of even and odd multiples of
+    8 other than y's, and orbital by orbital (each pointer may be aligned or not)."""
+    need_gpu()
+    shape, h = (16, 16, nx), 0.4
+    s = inputs.exchange_system(h=h, nocc=3, npsi=2, shape=shape, radius=1.5, seed=nx)
+    ctx = rsx.Context(shape, h, prec)
+    phi, psi = to_dev(s.phi, prec), to_dev(s.psi, prec)
+    ref = ctx.exchange_apply(phi, psi)
+    for kphi, kpsi, kout in ((1, 0, 0), (0, 1, 0), (0, 0, 1), (1, 1, 1)):
+        out = _off(torch.zeros_like(psi), kout)
+        got = ctx.exchange_apply(_off(phi, kphi), _off(psi, kpsi), out=out)
+        ctx.sync()
+        assert torch.equal(got, ref), (kphi, kpsi, kout)
+    V = ctx.poisson(phi[0] * phi[0])
+    rho = _off(phi[0] * phi[0], 1)
+    assert torch.equal(ctx.poisson(rho, V=_off(torch.zeros_like(V), 1)), V)
+    ctx.sync()
