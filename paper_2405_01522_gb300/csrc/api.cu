@@ -131,25 +131,7 @@ cudaError_t line_twiddles(rsx_ctx* c, int M, int lanes, void** out) {
 template <typename R>
 int make_tables(rsx_ctx* c) {
   const Geom& g = c->g;
-  // twiddles tw[t][k1] = exp(-2 pi i t k1 / M), t < 16, k1 < A, per axis (z, y, x)
   const int Ms[3] = {g.Mz, g.My, g.Mx};
-  const int As[3] = {g.Az, g.Ay, g.Ax};
-  for (int ax = 0; ax < 3; ++ax) {
-    std::vector<Cx<R>> tw(16 * As[ax]);
-    for (int t = 0; t < 16; ++t)
-      for (int k1 = 0; k1 < As[ax]; ++k1) {
-        const long long e = (long long)t * k1 % Ms[ax];
-        const double ang = 2.0 * M_PI * (double)e / (double)Ms[ax];
-        tw[t * As[ax] + k1].x = (R)cos(ang);
-        tw[t * As[ax] + k1].y = (R)(-sin(ang));
-      }
-    size_t have = 0;
-    int rc = grow(c, &c->tw[ax], &have, tw.size() * sizeof(Cx<R>), "twiddles");
-    if (rc) return rc;
-    rc = check_cuda(c, cudaMemcpy(c->tw[ax], tw.data(), tw.size() * sizeof(Cx<R>), cudaMemcpyHostToDevice),
-                    "twiddle upload");
-    if (rc) return rc;
-  }
   // kernel spectrum table
   const int hz = g.Mz / 2 + 1, hy = g.My / 2 + 1, hx = g.Mx / 2 + 1;
   const size_t nt = (size_t)hz * hy * hx;
@@ -177,6 +159,7 @@ int make_tables(rsx_ctx* c) {
       e = cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = line_twiddles<R>(c, g.Mz, p2_lanes<R>(g.Az), &c->twl);
     if (e == cudaSuccess) e = line_twiddles<R>(c, g.Mx, 8, &c->twx);
+    if (e == cudaSuccess && sizeof(R) == 4) e = line_twiddles<R>(c, g.Mz, 8, &c->twz8);   // Casida spectra
     if (e == cudaSuccess) e = launch_vhat_lanes<R>(g, (const R*)c->vhat, (R*)c->vlanes, 0);
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -468,7 +451,7 @@ int rsx_destroy(rsx_ctx* c) {
   cudaDeviceSynchronize();
   prof_collect(c);
   for (cudaEvent_t e : c->prof_pool) cudaEventDestroy(e);
-  void* bufs[] = {c->vhat, c->vlanes, c->twl, c->twx, c->tw[0], c->tw[1], c->tw[2], c->work, c->gscr, c->dsm, c->smallr, c->status,
+  void* bufs[] = {c->vhat, c->vlanes, c->twl, c->twx, c->twz8, c->work, c->gscr, c->dsm, c->smallr, c->status,
                   c->panel_hi, c->panel_lo, c->gemm_part, c->eig_work, c->gscr_kd, c->pos, c->tdhf_work, c->specw, c->ones};
   for (void* b : bufs)
     if (b) cudaFree(b);

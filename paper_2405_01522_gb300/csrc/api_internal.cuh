@@ -30,7 +30,7 @@ struct rsx_ctx {
   void* vlanes = nullptr;               // the same in pass 2's lane order (R, launch_vhat_lanes)
   void* twl = nullptr;                  // y/z line twiddles w_M^{-t k1}, t < lanes, k1 < M / lanes (R)
   void* twx = nullptr;                  // x line twiddles w_M^{-t k1}, t < 8, k1 < 2 Ax (R)
-  void* tw[3] = {nullptr, nullptr, nullptr};
+  void* twz8 = nullptr;                 // FP32: y/z line twiddles on 8 lanes (the Casida spectra)
   void* work = nullptr;   size_t work_bytes = 0;     // FFT intermediates
   void* gscr = nullptr;   size_t gscr_bytes = 0;     // pass-2 planes when shared memory is too small
   double* dsm = nullptr;  size_t dsm_bytes = 0;      // FP64 partials and small matrices

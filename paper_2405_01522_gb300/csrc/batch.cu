@@ -25,7 +25,6 @@
 #include "../../include/rsx.h"
 #include "api_internal.cuh"
 #include "dense.cuh"
-#include "poisson_kernels.cuh"
 
 using namespace rsx;
 

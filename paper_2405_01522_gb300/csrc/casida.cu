@@ -158,8 +158,7 @@ int casida_K_f32(rsx_ctx* c, const TSet* sets, int nsets, double* K, cudaStream_
   }
   if (rc) return rc;
   if (!c->specw) {   // panel weights, once per context
-    const size_t nw = (size_t)g.Hx * (g.My / 2 + 1) * (g.Mz / 2 + 1);
-    rc = grow(c, &c->specw, &c->specw_bytes, nw * sizeof(float), "panel weights");
+    rc = grow(c, &c->specw, &c->specw_bytes, spectrum_weight_elems(g) * sizeof(float), "panel weights");
     if (!rc)
       rc = check_cuda(c, launch_spectrum_weights(g, (const float*)c->vhat, (float)(c->h * c->h * c->h), (float*)c->specw, s),
                       "panel weights");
@@ -168,8 +167,7 @@ int casida_K_f32(rsx_ctx* c, const TSet* sets, int nsets, double* K, cudaStream_
   {
     ProfScope ps(c, kKSpectrum, s);
     rc = check_cuda(c,
-                    launch_spectrum_f32(g, nt, inter, (const Cx<float>*)c->tw[1], (const Cx<float>*)c->tw[0],
-                                        (const float*)c->specw, hi, lo, (size_t)ld, nrb, s),
+                    launch_spectrum_f32(g, nt, inter, (const Cx<float>*)c->twz8, (const float*)c->specw, hi, lo, nrb, s),
                     "spectrum panel");
   }
   if (rc) return rc;

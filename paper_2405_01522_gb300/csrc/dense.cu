@@ -525,11 +525,14 @@ __global__ void k_vhat_lanes(const R* __restrict__ T, int rows, int hz, int Az, 
 // host launchers
 
 template <typename R>
-cudaError_t launch_vhat_lanes(const Geom& g, const R* table, R* out, cudaStream_t s) {
+cudaError_t launch_lane_order(const Geom& g, const R* table, R* out, int lanes, cudaStream_t s) {
   const int rows = (g.Mx / 2 + 1) * (g.My / 2 + 1);
-  const int J = p2_lanes<R>(g.Az) == 8 ? line_j(g.Az) : 0;
-  k_vhat_lanes<R><<<1024, 256, 0, s>>>(table, rows, g.Mz / 2 + 1, g.Az, J, line_neg(g.Az), out);
+  k_vhat_lanes<R><<<1024, 256, 0, s>>>(table, rows, g.Mz / 2 + 1, g.Az, lanes == 8 ? line_j(g.Az) : 0, line_neg(g.Az), out);
   return cudaGetLastError();
+}
+template <typename R>
+cudaError_t launch_vhat_lanes(const Geom& g, const R* table, R* out, cudaStream_t s) {
+  return launch_lane_order<R>(g, table, out, p2_lanes<R>(g.Az), s);
 }
 
 cudaError_t launch_ghat(const Geom& g, double h, double scale, const double* cos_z, const double* cos_y,
@@ -853,6 +856,7 @@ cudaError_t launch_pair_products(const R* A, int na, const R* B, int nb, size_t 
 
 #define RSX_INST(R)                                                                                        \
   template cudaError_t launch_vhat_lanes<R>(const Geom&, const R*, R*, cudaStream_t);                     \
+  template cudaError_t launch_lane_order<R>(const Geom&, const R*, R*, int, cudaStream_t);                \
   template cudaError_t launch_gram<R>(const R*, int, const R*, int, size_t, double*, int, cudaStream_t,   \
                                       const R*, int*);                                                          \
   template cudaError_t launch_gram_reduce<R>(const double*, int, int, int, double, bool, double*, R*,      \

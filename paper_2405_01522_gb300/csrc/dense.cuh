@@ -12,6 +12,9 @@ cudaError_t launch_ghat(const Geom& g, double h, double scale, const double* cos
 // the kernel table in pass 2's lane order, (Mx/2+1)(My/2+1) rows of p2_row_factors<R>(Az) values (k_vhat_lanes)
 template <typename R>
 cudaError_t launch_vhat_lanes(const Geom& g, const R* table, R* out, cudaStream_t s);
+// any folded table [kx][|ky|][|kz|] in the lane order of the 8- or 16-lane split
+template <typename R>
+cudaError_t launch_lane_order(const Geom& g, const R* table, R* out, int lanes, cudaStream_t s);
 // part[blk][a][b] = partial sums of X_a(r) Y_b(r) w(r) (w may be null); na * nb <= 4096.
 // A kernel that gives up a bounded wait writes NaN partials and raises RSX_ETIMEOUT in *status.
 template <typename R>

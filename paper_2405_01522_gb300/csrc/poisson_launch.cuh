@@ -1,6 +1,5 @@
 // Launchers of the pair Poisson passes for one precision R (included once per TU).
 #pragma once
-#include "poisson_kernels.cuh"
 #include "poisson_pass2.cuh"
 
 namespace rsx {
@@ -21,12 +20,6 @@ inline int max_dyn_smem() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   return v;
-}
-
-// the spectrum kernel's work plane and line scratch (nt threads, 16 lanes per line)
-inline size_t spectrum_smem(const Geom& g, int nt) {
-  const int A = g.Ay > g.Az ? g.Ay : g.Az;
-  return sizeof(Cx<float>) * ((size_t)(nt / 16) * A * kScrPitch + (size_t)g.nz * (g.My + 1));
 }
 
 // ---- pass 2 (k_pass2): the plane in shared memory where it fits beside the line scratch

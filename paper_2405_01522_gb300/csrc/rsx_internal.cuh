@@ -8,13 +8,20 @@
 
 namespace rsx {
 
-// Line transforms: an FFT of length M = 16 * A along one axis is done by a half-warp
-// (16 lanes) in two register stages: A-point DFTs over stride-16 inputs, a twiddle,
-// a transpose through shared memory, then 16-point DFTs (see poisson_kernels.cuh).
-constexpr int kLinesPerCta = 16;      // 8 warps x 2 half-warps
-constexpr int kThreads = 256;
-constexpr int kScrPitch = 17;         // scratch row pitch (complex), avoids bank conflicts
-constexpr int kRowsPerCta = 32;       // rows (y) per CTA in the x passes
+// The pair Poisson solve by pruned, zero-padded FFT convolution.  The potential of a pair
+// density rho = f1 f2 on the box (nz, ny, nx) is
+//     V = h^3/N_pad * IDFT( ghat * DFT(rho zero-padded to (2nz, 2ny, 2nx)) )
+// restricted to the box (Sec. 3.1: Eq. 2's integral as a Poisson problem at O(N log N); padding
+// twice the box makes the periodic convolution the isolated one).  Three passes:
+//   pass 1  x forward, real-to-complex (two rows y, y+1 packed as one complex line), output
+//           I[q][kx][z][y], kx in [0, Mx/2]: (Mx/2+1) nz ny complex      (poisson_xpass.cuh)
+//   pass 2  per (q, kx): y forward on nz rows, z forward + multiply by ghat + z inverse on My
+//           columns, y inverse keeping y < ny; in place on I             (poisson_pass2.cuh)
+//   pass 3  per output p: x inverse complex-to-real of every pair of p's list, keeping x < nx,
+//           and out_p -= partner * V (Eq. 2's sum over j)                (poisson_xpass.cuh)
+// Only nz of the 2nz z-planes and ny of the 2ny rows are non-zero, so the x transforms run on
+// nz ny rows and the y transforms on nz rows per kx; I is 4x smaller than a padded half
+// spectrum.  The line transforms are in poisson_lines.cuh.
 
 // Which pair densities a batch holds and which pairs each output accumulates.
 //   PROD: pair q = b * na + a  has density A[a] * B[b]  (exchange: A = phi, B = psi;
@@ -125,12 +132,13 @@ template <typename R>
 cudaError_t launch_pass3(const Geom& g, const PairMap<R>& pm, int q0, int p0, int np, int pot, const Cx<R>* inter,
                          const Cx<R>* twx, R* out, cudaStream_t s);
 // forward y/z transform of each pair plane, weighted by sqrt(w_G vhat(G) h^3) and split
-// into bf16 hi/lo of the K panel, tile-major [ld/64][nrb][128][64] (nrb row blocks of 128)
-cudaError_t launch_spectrum_f32(const Geom& g, int nq, const Cx<float>* inter, const Cx<float>* twy,
-                                const Cx<float>* twz, const float* wsq, uint16_t* hi,
-                                uint16_t* lo, size_t ld, int nrb, cudaStream_t s);
-// panel weights wsq = sqrt(w_kx vhat h^3) on the folded half spectrum (Hx, My/2+1, Mz/2+1)
-cudaError_t launch_spectrum_weights(const Geom& g, const float* vhat, float h3, float* wsq, cudaStream_t s);
+// into bf16 hi/lo of the K panel, tile-major [ld/64][nrb][128][64] (nrb row blocks of 128).
+// tw8: w_M^{-t k1}, t < 8, k1 < M / 8; wl: launch_spectrum_weights
+cudaError_t launch_spectrum_f32(const Geom& g, int nq, const Cx<float>* inter, const Cx<float>* tw8,
+                                const float* wl, uint16_t* hi, uint16_t* lo, int nrb, cudaStream_t s);
+// panel weights sqrt(w_kx vhat h^3) in lane order, spectrum_weight_elems(g) floats
+size_t spectrum_weight_elems(const Geom& g);
+cudaError_t launch_spectrum_weights(const Geom& g, const float* vhat, float h3, float* wl, cudaStream_t s);
 template <typename R>
 size_t pass2_smem_bytes(const Geom& g, bool* fits);
 template <typename R>
