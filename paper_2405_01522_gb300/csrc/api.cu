@@ -170,6 +170,14 @@ int make_tables(rsx_ctx* c) {
 }
 
 template <typename R>
+int prepare_passes(rsx_ctx* c) {
+  cudaError_t e = prepare_pass1<R>(c->g);
+  if (e == cudaSuccess) e = prepare_pass2<R>(c->g, &c->p2_ctas);
+  if (e == cudaSuccess) e = prepare_pass3<R>(c->g);
+  return check_cuda(c, e, "kernel attributes");
+}
+
+template <typename R>
 PairMap<R> pair_map(int mode, const void* A, const void* B, int na, int nb, size_t N) {
   PairMap<R> pm;
   pm.mode = mode;
@@ -214,8 +222,7 @@ int solve_pairs(rsx_ctx* c, const PairMap<R>& pm, int q0, int nq, int p0, int np
   int grid;
   R* gscr = nullptr;
   if (fits) {
-    const int per_sm = c->pass2_ctas_per_sm<R>();
-    grid = (int)std::min<long long>(nwork, (long long)per_sm * c->nsm);
+    grid = (int)std::min<long long>(nwork, (long long)c->p2_ctas * c->nsm);
   } else {
     grid = (int)std::min<long long>(nwork, 2LL * c->nsm);
     rc = grow(c, &c->gscr, &c->gscr_bytes, pass2_gscratch_bytes<R>(g, grid), "pass-2 plane scratch");
@@ -418,6 +425,7 @@ int rsx_create(rsx_ctx** out, int nz, int ny, int nx, double h, int precision, i
   if (const char* e = getenv("RSX_PASS1_GROUP")) g.p1_group = atoi(e) > 0 ? atoi(e) : 0;
   g.p2_global = 0;
   cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, device);
+  cudaDeviceGetAttribute(&g.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
   c->work_limit = std::min<size_t>((size_t)(0.4 * (double)freeb), (size_t)64 << 30);
@@ -429,7 +437,8 @@ int rsx_create(rsx_ctx** out, int nz, int ny, int nx, double h, int precision, i
 #ifdef RSX_CHECKED
   g.dbg = c->status;   // out-of-range indices of the FFT passes are reported here
 #endif
-  const int rc = precision == RSX_FP32 ? make_tables<float>(c) : make_tables<double>(c);
+  int rc = precision == RSX_FP32 ? make_tables<float>(c) : make_tables<double>(c);
+  if (!rc) rc = precision == RSX_FP32 ? prepare_passes<float>(c) : prepare_passes<double>(c);
   if (rc) {
     rsx_destroy(c);
     return rc;

@@ -45,7 +45,7 @@ struct rsx_ctx {
   void* specw = nullptr; size_t specw_bytes = 0;         // Casida panel weights (float)
   void* ones = nullptr; size_t ones_bytes = 0;           // unit field (R), Poisson solves of a density
   void* tdhf_work = nullptr; size_t tdhf_work_bytes = 0; // full TDHF: L, A + B, products
-  int p2_occ[2] = {0, 0};
+  int p2_ctas = 1;   // resident CTAs per SM of pass 2's shared-memory variant
   int p2_threads = 256, p2_lanes = 16;   // tuning knobs kept for callers (no effect, see rsx.h)
   int chunk_outputs = 0;   // tuning: output orbitals per exchange chunk (0 = as many as fit)
   long long wait_limit = -1;   // spin rounds of the bounded grid waits (-1: the kernels' default)
@@ -63,12 +63,6 @@ struct rsx_ctx {
   char err[512] = {0};
 
   size_t elem_size() const { return precision == 1 ? 4 : 8; }
-  template <typename R>
-  int pass2_ctas_per_sm() {
-    int& o = p2_occ[sizeof(R) == 8 ? 1 : 0];
-    if (o == 0) o = std::max(1, rsx::pass2_occupancy<R>(g));
-    return o;
-  }
 };
 
 namespace rsx {

@@ -125,7 +125,7 @@ int record(rsx_batch* b, cudaStream_t s) {
     rc = bcuda(b, launch_pass1<float>(c->g, pm, 0, grp.npairs, inter, twx, s), "batch pass 1");
     if (rc) return rc;
     const long long nwork = (long long)grp.npairs * c->g.Hx;
-    const int grid = (int)std::min<long long>(nwork, (long long)c->pass2_ctas_per_sm<float>() * c->nsm);
+    const int grid = (int)std::min<long long>(nwork, (long long)c->p2_ctas * c->nsm);
     rc = bcuda(b, launch_pass2<float>(c->g, grp.npairs, inter, (const Cx<float>*)c->twl, (const float*)c->vlanes, nullptr, grid, s),
                "batch pass 2");
     if (rc) return rc;

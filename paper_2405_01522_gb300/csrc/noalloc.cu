@@ -83,8 +83,7 @@ int exchange_noalloc(rsx_ctx* c, const void* phi, int nocc, const void* psi, int
   pm.N = N;
   Cx<R>* inter = (Cx<R>*)scratch;
   const Cx<R>* twx = (const Cx<R>*)c->twx;
-  const int per_sm = std::max(1, pass2_occupancy<R>(g));
-  const int grid = (int)std::min<long long>((long long)nocc * g.Hx, (long long)per_sm * c->nsm);
+  const int grid = (int)std::min<long long>((long long)nocc * g.Hx, (long long)c->p2_ctas * c->nsm);
   for (int p = 0; p < npsi; ++p) {
     int rc = check_cuda(c, launch_pass1<R>(g, pm, p * nocc, nocc, inter, twx, s), "noalloc pass 1");
     if (rc) return rc;

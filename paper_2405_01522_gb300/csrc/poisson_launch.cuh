@@ -15,11 +15,9 @@ inline bool axis_supported_impl(int A) {
   }
 }
 
-inline int max_dyn_smem() {
-  int dev = 0, v = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return v;
+template <class K>
+inline cudaError_t set_smem(K k, size_t bytes) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // ---- pass 2 (k_pass2): the plane in shared memory where it fits beside the line scratch
@@ -37,7 +35,7 @@ size_t pass2_smem_bytes(const Geom& g, bool* fits) {
 #undef RSX_CASE
     default: break;
   }
-  const bool f = g.p2_global == 0 && sc + pl <= (size_t)max_dyn_smem();
+  const bool f = g.p2_global == 0 && sc + pl <= (size_t)g.smem_optin;
   if (fits) *fits = f;
   return f ? sc + pl : sc;
 }
@@ -56,27 +54,32 @@ inline auto pass2_kernel(bool dsmem) {
   return k_pass2<R, A, false>;
 }
 
+// both variants (a context may switch p2_global)
 template <typename R>
-int pass2_occupancy(const Geom& g) {
+cudaError_t prepare_pass2(const Geom& g, int* ctas) {
+  Geom gs = g;
+  gs.p2_global = 0;
   bool fits = false;
-  const size_t smem = pass2_smem_bytes<R>(g, &fits);
-  int nb = 1;
+  const size_t smem = pass2_smem_bytes<R>(gs, &fits);
+  gs.p2_global = 1;
+  const size_t smem_g = pass2_smem_bytes<R>(gs, nullptr);
+  *ctas = 1;
   switch (g.Ay) {
-#define RSX_CASE(a)                                                                                       \
-  case a: {                                                                                               \
-    auto k = pass2_kernel<R, a>(fits);                                                                    \
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess || \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, p2_threads<R>(a), smem) != cudaSuccess) { \
-      cudaGetLastError();                                                                                 \
-      nb = 1;                                                                                             \
-    }                                                                                                     \
-    break;                                                                                                \
+#define RSX_CASE(a)                                                                                            \
+  case a: {                                                                                                    \
+    cudaError_t e = set_smem(pass2_kernel<R, a>(false), smem_g);                                               \
+    if (e != cudaSuccess || !fits) return e;                                                                   \
+    auto k = pass2_kernel<R, a>(true);                                                                         \
+    e = set_smem(k, smem);                                                                                     \
+    int nb = 0;                                                                                                \
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, p2_threads<R>(a), smem);   \
+    *ctas = nb > 0 ? nb : 1;                                                                                   \
+    return e;                                                                                                  \
   }
     RSX_FOR_EACH_A(RSX_CASE)
 #undef RSX_CASE
-    default: break;
+    default: return cudaErrorInvalidValue;
   }
-  return nb;
 }
 
 template <typename R>
@@ -91,8 +94,6 @@ cudaError_t launch_pass2(const Geom& g, int nq, Cx<R>* inter, const Cx<R>* twl, 
 #define RSX_CASE(a)                                                                                  \
   case a: {                                                                                          \
     auto k = pass2_kernel<R, a>(fits);                                                               \
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-    if (e != cudaSuccess) return e;                                                                  \
     k<<<grid, p2_threads<R>(a), smem, s>>>(g, nq, inter, twl, vlanes, (Cx<R>*)gscratch);           \
     return cudaGetLastError();                                                                       \
   }

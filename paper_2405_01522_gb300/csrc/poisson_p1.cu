@@ -4,6 +4,25 @@
 
 namespace rsx {
 
+template <typename R, int A>
+constexpr size_t pass1_smem() {
+  using X = XWarp<R, A>;
+  return sizeof(Cx<R>) * kXWarps * (size_t)(X::SCR > X::TILE ? X::SCR : X::TILE);
+}
+
+template <typename R>
+cudaError_t prepare_pass1(const Geom& g) {
+  switch (g.Ax) {
+#define RSX_CASE(a) \
+  case a: return set_smem(k_pass1<R, a>, pass1_smem<R, a>());
+    RSX_FOR_EACH_A(RSX_CASE)
+#undef RSX_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t prepare_pass1<float>(const Geom&);
+template cudaError_t prepare_pass1<double>(const Geom&);
+
 template <typename R>
 cudaError_t launch_pass1(const Geom& g, const PairMap<R>& pm, int q0, int nq, Cx<R>* inter,
                          const Cx<R>* twx, cudaStream_t s) {
@@ -17,11 +36,8 @@ cudaError_t launch_pass1(const Geom& g, const PairMap<R>& pm, int q0, int nq, Cx
   switch (g.Ax) {
 #define RSX_CASE(a)                                                                                  \
   case a: {                                                                                          \
-    using X = XWarp<R, a>;                                                                           \
-    const size_t smem = sizeof(Cx<R>) * kXWarps * (size_t)(X::SCR > X::TILE ? X::SCR : X::TILE);     \
+    const size_t smem = pass1_smem<R, a>();                                                           \
     auto k = k_pass1<R, a>;                                                                          \
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-    if (e != cudaSuccess) return e;                                                                  \
     k<<<(unsigned)nblk, 32 * kXWarps, smem, s>>>(gg, pm, q0, nq, inter, twx);                        \
     return cudaGetLastError();                                                                       \
   }

@@ -4,6 +4,25 @@
 
 namespace rsx {
 
+template <typename R, int A>
+constexpr size_t pass3_smem() {
+  using X = XWarp<R, A>;
+  return sizeof(Cx<R>) * kXWarps * (size_t)(X::SCR + X::TILE);
+}
+
+template <typename R>
+cudaError_t prepare_pass3(const Geom& g) {
+  switch (g.Ax) {
+#define RSX_CASE(a) \
+  case a: return set_smem(k_pass3<R, a>, pass3_smem<R, a>());
+    RSX_FOR_EACH_A(RSX_CASE)
+#undef RSX_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t prepare_pass3<float>(const Geom&);
+template cudaError_t prepare_pass3<double>(const Geom&);
+
 template <typename R>
 cudaError_t launch_pass3(const Geom& g, const PairMap<R>& pm, int q0, int p0, int np, int pot, const Cx<R>* inter,
                          const Cx<R>* twx, R* out, cudaStream_t s) {
@@ -13,11 +32,8 @@ cudaError_t launch_pass3(const Geom& g, const PairMap<R>& pm, int q0, int p0, in
   switch (g.Ax) {
 #define RSX_CASE(a)                                                                                  \
   case a: {                                                                                          \
-    using X = XWarp<R, a>;                                                                           \
-    const size_t smem = sizeof(Cx<R>) * kXWarps * (size_t)(X::SCR + X::TILE);                        \
+    const size_t smem = pass3_smem<R, a>();                                                           \
     auto k = k_pass3<R, a>;                                                                          \
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-    if (e != cudaSuccess) return e;                                                                  \
     k<<<(unsigned)nblk, 32 * kXWarps, smem, s>>>(g, pm, q0, p0, np, pot, inter, twx, out);           \
     return cudaGetLastError();                                                                       \
   }

@@ -95,6 +95,7 @@ struct Geom {
   int Mz, My, Mx;     // padded (2n)
   int Az, Ay, Ax;     // M / 16
   int Hx;             // Mx / 2 + 1 (half spectrum along x)
+  int smem_optin;     // shared memory a CTA may opt into on the context's device (bytes)
   int p1_group;       // tuning: pass-1 block order (0: pair-major; G > 0: pairs fastest in groups of G)
   int p2_global;      // tuning: 1 = the y/z pass keeps its work plane in global scratch even where
                       // shared memory would hold it (0 = shared memory whenever it fits)
@@ -118,6 +119,16 @@ __device__ inline bool in_range_checked(int* dbg, long long i, long long n) {
 #else
 #define RSX_IN_RANGE(g, i, n) true
 #endif
+
+// Kernel attributes of the three passes for geometry g on the current device (once per context:
+// the launchers below make no attribute calls).  ctas: resident CTAs per SM of pass 2's
+// shared-memory variant.
+template <typename R>
+cudaError_t prepare_pass1(const Geom& g);
+template <typename R>
+cudaError_t prepare_pass2(const Geom& g, int* ctas);
+template <typename R>
+cudaError_t prepare_pass3(const Geom& g);
 
 // ---- launchers (defined per precision in poisson_f32.cu / poisson_f64.cu)
 template <typename R>
@@ -143,9 +154,6 @@ template <typename R>
 size_t pass2_smem_bytes(const Geom& g, bool* fits);
 template <typename R>
 size_t pass2_gscratch_bytes(const Geom& g, int grid);   // global plane scratch of a launch of `grid` CTAs
-template <typename R>
-int pass2_occupancy(const Geom& g);  // resident pass-2 CTAs per SM (shared-memory variant)
-
 bool axis_supported(int A);
 
 }  // namespace rsx

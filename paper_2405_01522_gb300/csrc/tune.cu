@@ -89,7 +89,6 @@ void apply(rsx_ctx* c, const rsx_tuning& t) {
   c->p2_lanes = t.p2_lanes;
   c->g.p1_group = t.p1_group;
   c->g.p2_global = t.p2_global;
-  c->p2_occ[0] = c->p2_occ[1] = 0;
   c->chunk_outputs = t.chunk_outputs;
 }
 
