@@ -206,6 +206,7 @@ int solve_pairs(rsx_ctx* c, const PairMap<R>& pm, int q0, int nq, int p0, int np
                 int pot) {
   Geom g = c->g;
   g.dbg_nq = nq;   // pairs of this launch's intermediate (read by bounds-checked builds)
+  g.pdl = (long long)nq * g.Hx <= c->nsm;   // at most one plane per SM: launch latency (launch_pdl)
   const size_t need = (size_t)nq * g.inter_elems() * sizeof(Cx<R>);
   int rc = grow(c, &c->work, &c->work_bytes, need, "FFT intermediates");
   if (rc) return rc;

@@ -1,5 +1,7 @@
 // Launchers of the pair Poisson passes for one precision R (included once per TU).
 #pragma once
+#include <utility>
+
 #include "poisson_pass2.cuh"
 
 namespace rsx {
@@ -18,6 +20,27 @@ inline bool axis_supported_impl(int A) {
 template <class K>
 inline cudaError_t set_smem(K k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// Launch, with programmatic stream serialisation (see pdl_wait) when pdl is set.  It pays where
+// the passes are launch latency: a 32^3 Poisson solve takes 7.5 us instead of 14.3 in stream
+// order.  Where every SM has work it costs: CTAs set up early take their places while the
+// kernel before still runs, and the persistent pass 2 ends up unevenly dealt (96^3 x 512
+// pairs 6.76 -> 6.89 ms, FP64 32^3 x 16 279 -> 349 us, the uneven batch 4.44 -> 4.75 ms); the
+// line lies at one plane of pass 2 per SM (solve_pairs).
+template <class... P, class... Q>
+inline cudaError_t launch_pdl(bool pdl, void (*k)(P...), long long grid, int block, size_t smem, cudaStream_t s, Q&&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<Q>(args)...);
 }
 
 // ---- pass 2 (k_pass2): the plane in shared memory where it fits beside the line scratch
@@ -94,8 +117,7 @@ cudaError_t launch_pass2(const Geom& g, int nq, Cx<R>* inter, const Cx<R>* twl, 
 #define RSX_CASE(a)                                                                                  \
   case a: {                                                                                          \
     auto k = pass2_kernel<R, a>(fits);                                                               \
-    k<<<grid, p2_threads<R>(a), smem, s>>>(g, nq, inter, twl, vlanes, (Cx<R>*)gscratch);           \
-    return cudaGetLastError();                                                                       \
+    return launch_pdl(g.pdl, k, grid, p2_threads<R>(a), smem, s, g, nq, inter, twl, vlanes, (Cx<R>*)gscratch); \
   }
     RSX_FOR_EACH_A(RSX_CASE)
 #undef RSX_CASE

@@ -18,6 +18,13 @@
 
 namespace rsx {
 
+// Programmatic dependent launch: the passes are launched so that a kernel's CTAs may be set up
+// while the kernel before it in the stream drains.  Every pass starts with pdl_wait(), before
+// its first access to memory that kernel touches (it returns when that kernel is complete
+// and its writes are visible), and lets its own successor be set up from its start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __host__ __device__ constexpr int line_tw_count(int A, int neg) { return neg - 1 > 2 * A - neg ? neg - 1 : 2 * A - neg; }
 __host__ __device__ constexpr int line_neg(int A) {   // 2A: no negative rows
   int best = 2 * A;

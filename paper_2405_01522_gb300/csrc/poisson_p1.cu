@@ -38,8 +38,7 @@ cudaError_t launch_pass1(const Geom& g, const PairMap<R>& pm, int q0, int nq, Cx
   case a: {                                                                                          \
     const size_t smem = pass1_smem<R, a>();                                                           \
     auto k = k_pass1<R, a>;                                                                          \
-    k<<<(unsigned)nblk, 32 * kXWarps, smem, s>>>(gg, pm, q0, nq, inter, twx);                        \
-    return cudaGetLastError();                                                                       \
+    return launch_pdl(gg.pdl, k, nblk, 32 * kXWarps, smem, s, gg, pm, q0, nq, inter, twx);                   \
   }
     RSX_FOR_EACH_A(RSX_CASE)
 #undef RSX_CASE

@@ -34,8 +34,7 @@ cudaError_t launch_pass3(const Geom& g, const PairMap<R>& pm, int q0, int p0, in
   case a: {                                                                                          \
     const size_t smem = pass3_smem<R, a>();                                                           \
     auto k = k_pass3<R, a>;                                                                          \
-    k<<<(unsigned)nblk, 32 * kXWarps, smem, s>>>(g, pm, q0, p0, np, pot, inter, twx, out);           \
-    return cudaGetLastError();                                                                       \
+    return launch_pdl(g.pdl, k, nblk, 32 * kXWarps, smem, s, g, pm, q0, p0, np, pot, inter, twx, out);      \
   }
     RSX_FOR_EACH_A(RSX_CASE)
 #undef RSX_CASE

@@ -94,7 +94,9 @@ __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
   const int lrow = LN == 8 && (line | 7) < NL ? (line & ~7) | ((line >> 1) & 3) | ((line & 1) << 2) : line;
   Cx<R>* sc = scr + line * S::SCR;
   typename S::Tw tw;
-  tw.init(twg, t);
+  tw.init(twg, t);   // tables are written once, by rsx_create
+  pdl_launch();
+  pdl_wait();
   const int Hy = M / 2 + 1;
   const int nplane = NB * NB;
   const int nwork = nq * g.Hx;

@@ -103,7 +103,9 @@ __global__ void __launch_bounds__(32 * kXWarps, p1_min_ctas<R>(A)) k_pass1(Geom 
     ql = (b / nob) * g.p1_group + lo;
   }
   const int oct = ob * kXWarps + warp;
+  pdl_launch();
   if (ql >= nq || oct >= noct) return;   // whole warps: the last group, the last block
+  pdl_wait();
   const R *f1, *f2;
   pm.pair(q0 + ql, f1, f2);
   const size_t base = (size_t)oct * 8 * NB;
@@ -187,7 +189,9 @@ __global__ void __launch_bounds__(32 * kXWarps, p3_min_ctas<R>(A)) k_pass3(Geom 
   // outputs are the fastest index: the CTAs in flight share their rows, so the partner rows
   // they multiply come from HBM once and then from L2 for the other outputs
   const int pl = (int)(blockIdx.x % np), oct = (int)(blockIdx.x / np) * kXWarps + warp;
+  pdl_launch();
   if (oct >= g.nz * (g.ny / 8)) return;   // whole warps
+  pdl_wait();
   const int p = p0 + pl;
   const size_t base = (size_t)oct * 8 * NB;
   if (!RSX_IN_RANGE(g, base + 8 * NB - 1, g.N())) return;

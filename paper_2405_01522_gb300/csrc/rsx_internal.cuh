@@ -100,6 +100,7 @@ struct Geom {
   int p2_global;      // tuning: 1 = the y/z pass keeps its work plane in global scratch even where
                       // shared memory would hold it (0 = shared memory whenever it fits)
   int* dbg = nullptr; // bounds-checked builds: the status word an out-of-range index is reported in
+  bool pdl = false;   // launch the passes with programmatic stream serialisation (launch_pdl)
   int dbg_nq = 0;     // bounds-checked builds: pairs the launch's intermediate holds (0: unknown)
   __host__ __device__ size_t N() const { return (size_t)nz * ny * nx; }
   __host__ __device__ size_t inter_elems() const { return (size_t)Hx * nz * ny; }  // complex per pair

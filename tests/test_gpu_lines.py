@@ -61,3 +61,48 @@ def test_x_passes_off_sixteen_byte_boundaries(prec, nx):
     rho = _off(phi[0] * phi[0], 1)
     assert torch.equal(ctx.poisson(rho, V=_off(torch.zeros_like(V), 1)), V)
     ctx.sync()
+
+
+@pytest.mark.parametrize("edge,prec", [(16, "fp32"), (32, "fp32"), (32, "fp64")])
+def test_back_to_back_small_solves(edge, prec):
+    """Solves of at most one plane per SM are launched so that a pass's CTAs may be set up while
+    the kernel before it drains.  A chain of them, each reading what a torch kernel made of the
+    last result and overwriting the library's and the caller's buffers, gives the bits of the
+    same chain with a synchronisation after every step; also when replayed from a CUDA graph."""
+    need_gpu()
+    shape, h = (edge,) * 3, 0.4
+    s = inputs.exchange_system(h=h, nocc=1, npsi=1, shape=shape, radius=1.5, seed=edge)
+    ctx = rsx.Context(shape, h, prec)
+    phi = to_dev(s.phi, prec)
+
+    def chain(sync):
+        rho = (phi[0] * phi[0]).contiguous()
+        V, seen = torch.empty_like(rho), []
+        for k in range(12):
+            ctx.poisson(rho, V=V)
+            if sync:
+                torch.cuda.synchronize()
+            rho.mul_(0.5).add_(V, alpha=0.05)          # in place: the next solve's input
+            ctx.exchange_apply(phi, rho.unsqueeze(0), out=V.unsqueeze(0))
+            if sync:
+                torch.cuda.synchronize()
+            rho.sub_(V, alpha=0.1)
+            seen.append(rho.clone())
+        torch.cuda.synchronize()
+        return seen
+
+    ref = chain(True)
+    for a, b in zip(ref, chain(False)):
+        assert torch.equal(a, b)
+    rho, V = (phi[0] * phi[0]).contiguous(), torch.empty_like(phi[0])
+    want = ctx.poisson(rho).clone()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        ctx.poisson(rho, V=V)
+        ctx.poisson(rho, V=V)
+    V.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(V, want)
