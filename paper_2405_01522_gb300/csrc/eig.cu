@@ -2,10 +2,11 @@
 // with B = 0 the problem A X = omega X is Hermitian; only the lowest roots are needed).
 //
 //   k_tda_assemble    A = diag(eps_a - eps_i) + delta_M K - K_d, symmetrised
-//   k_tridiag_cluster Householder reduction A = Q T Q^T on one thread-block cluster with the
-//                     matrix in distributed shared memory (n up to ~530); k_tridiag_coop the
-//                     cooperative multi-CTA form for larger n; k_tridiagonalise one CTA
-//                     (reflectors kept in A in every form)
+//   k_tridiag_regs    Householder reduction A = Q T Q^T in FP32 on one thread-block cluster with
+//                     the matrix in registers (n <= 768); k_tridiag_cluster the same with the
+//                     matrix in distributed shared memory (FP32 n up to ~900, FP64 ~630);
+//                     k_tridiag_coop the cooperative multi-CTA form for larger n;
+//                     k_tridiagonalise one CTA (reflectors kept in A in every form)
 //   k_multisect       lowest nroots eigenvalues of T by Sturm-count multisection (a warp
 //                     per root)
 //   k_invit           inverse iteration on T (a warp per root); k_invit_clusters redoes
@@ -18,10 +19,12 @@
 #include <algorithm>
 #include <cstdlib>
 #include <string>
+#include <type_traits>
 
 #include "../../include/rsx.h"
 #include "api_internal.cuh"
 #include "eig.cuh"
+#include "eig_tridiag_regs.cuh"
 
 namespace rsx {
 namespace {
@@ -824,6 +827,47 @@ static int tridiagonalise(rsx_ctx* c, F* A, int n, F* d, F* e, F* tau, F* scr, F
     }
     return check_cuda(c, cudaLaunchKernelEx(&cfg, kern, A, n, d, e, tau), "cluster tridiagonalisation");
   };
+  // FP32, n <= 768: the rows in the registers of a 16-CTA cluster, 16, 32 or 48 rows per CTA (the
+  // smallest that holds n; 64 would need more registers than a thread has).  Faster at every
+  // size it takes: n = 96 0.64 -> 0.52 ms a solve, 256 1.30 -> 0.87, 512 2.80 -> 1.73,
+  // 768 5.30 -> 3.29
+  auto try_regs = [&](auto nl) -> int {
+    constexpr int NL = decltype(nl)::value;
+    auto kern = k_tridiag_regs<NL>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(TridiagRegs<NL>::CS);
+    cfg.blockDim = dim3(TridiagRegs<NL>::NT);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = TridiagRegs<NL>::CS;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int ncl = 0;
+    if (cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg) != cudaSuccess || ncl < 1) {
+      cudaGetLastError();
+      return -1;
+    }
+    return check_cuda(c, cudaLaunchKernelEx(&cfg, kern, A, n, d, e, tau, c->status), "cluster tridiagonalisation");
+  };
+  if constexpr (sizeof(F) == 4) {
+    if (force.empty() && n >= 64) {
+      int r = -1;
+      if (n <= 256)
+        r = try_regs(std::integral_constant<int, 16>{});
+      else if (n <= 512)
+        r = try_regs(std::integral_constant<int, 32>{});
+      else if (n <= 768)
+        r = try_regs(std::integral_constant<int, 48>{});
+      if (r >= 0) return r;
+    }
+  }
   if (force.empty() || force == "cluster")
     for (int CS : {16, 8}) {
       const int r = try_cluster(CS, false);
