@@ -77,15 +77,25 @@ __global__ void k_ham_apply(const float* __restrict__ f, int nb, int n, float in
 
 // The same operator by z-marching tiles: a block owns kHamTy rows y of 4-point float4
 // columns along x (one per thread) for kHamZc consecutive planes z.  Each thread keeps
-// its column's planes z-2 .. z+2 in registers (and z+3, loaded a plane ahead of its use,
-// like every other global load of the loop); the plane z rows y0-2 .. y0+kHamTy+1 are
+// its column's planes z-2 .. z+3 in registers; the plane z rows y0-2 .. y0+kHamTy+1 are
 // staged in shared memory (with one zero float4 on each side in x) for the x and y
-// neighbours.  One global load per point instead of thirteen; the arithmetic per point
-// is that of k_ham_apply, term by term.  n % 4 == 0, every array 16-byte aligned.
-// With jr given, the output is one damped Jacobi sweep on (H) x = jr instead (H with
+// neighbours, in two buffers, so that a plane needs one barrier.  One global load per point
+// instead of thirteen; the stencil is that of k_ham_apply, term by term.  n % 4 == 0, every
+// array 16-byte aligned.
+// With HJ, the output is one damped Jacobi sweep on (H) x = jr instead (H with
 // V = 0 and the shift T_b): out = f + omega (jr - H f) / (d0 + T_b), the arithmetic of
 // k_ke_jacobi.
-constexpr int kHamTy = 8;
+//
+// Bound by memory latency: every global load, the operands V, mask and jr among them, is
+// issued a plane or more ahead of its use, and the operands that a call does not have are
+// compiled out of its registers.  Four rows: each thread loads exactly one halo row, and
+// 8 rows leave fewer blocks in flight (43 us below; 12 rows 45).  3 blocks of 256 threads an
+// SM: 2 or 4 (spills) measured 39.0 and 37.5 us.  12 planes: 8 to 16 are the same, 24 slower
+// at n = 64 (17 against 14 us).
+// 96^3, 16 bands (113 MB, 17 us at the copy rate): H 53 -> 35 us, a sweep 60 -> 44 us; H at
+// 128^3 109 -> 74 us, at 64^3 19.7 -> 13.9.  A multiplication by omega / (d0 + T_b) would take
+// 4 us off a sweep, but its rounding turns the sign of an orbital now and then.
+constexpr int kHamTy = 4;
 constexpr int kHamZc = 12;
 
 __device__ __forceinline__ float ham_point(float c, float xm2, float xm1, float xp1, float xp2, float ym2,
@@ -103,86 +113,90 @@ __device__ __forceinline__ float ham_point(float c, float xm2, float xm1, float 
   return -0.5f * lap * inv12h2;
 }
 
-__global__ void __launch_bounds__(512) k_ham_apply_z(const float* __restrict__ f, int n, float inv12h2,
-                                                     const float* __restrict__ V, const double* __restrict__ shift,
-                                                     const float* __restrict__ mask, const float* __restrict__ jr,
-                                                     float d0, float omega, float* __restrict__ out) {
-  extern __shared__ float4 hs4[];   // [kHamTy + 4][n/4 + 2]
-  const int n4 = n >> 2, W = n4 + 2;
+template <bool HV, bool HM, bool HJ>
+__global__ void __launch_bounds__(256, 3) k_ham_apply_z(const float* __restrict__ f, int n, float inv12h2,
+                                                        const float* __restrict__ V, const double* __restrict__ shift,
+                                                        const float* __restrict__ mask, const float* __restrict__ jr,
+                                                        float d0, float omega, float* __restrict__ out) {
+  extern __shared__ float4 hs4[];   // [2][kHamTy + 4][n/4 + 2]
+  const int n4 = n >> 2, W = n4 + 2, nn4 = n * n4;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int y0 = blockIdx.x * kHamTy, y = y0 + ty;
+  const int y0 = blockIdx.x * kHamTy, y = y0 + ty;   // y < n: n % 4 == 0 and four rows a block
   const int z0 = blockIdx.y * kHamZc, z1 = min(z0 + kHamZc, n);
   const int b = blockIdx.z;
-  const size_t nn4 = (size_t)n * n4, N4 = nn4 * n;
-  const float4* f4 = reinterpret_cast<const float4*>(f) + (size_t)b * N4;
+  const size_t band = (size_t)b * nn4 * n;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto ld = [&](int yy, int zz) {
-    return (yy >= 0 && yy < n && zz >= 0 && zz < n) ? __ldg(f4 + (size_t)zz * nn4 + (size_t)yy * n4 + tx) : zero;
-  };
-  for (int r = ty; r < kHamTy + 4; r += kHamTy) {   // x halo: zeros, never overwritten
+  const int yh = ty < 2 ? y0 - 2 + ty : y0 + ty + 2;   // this thread's halo row
+  const bool acth = yh >= 0 && yh < n;
+  const int col = y * n4 + tx, colh = yh * n4 + tx;
+  const float4* f4 = reinterpret_cast<const float4*>(f) + band;
+  auto ld = [&](int z, int c) { return z >= 0 && z < n ? __ldg(f4 + ((ptrdiff_t)z * nn4 + c)) : zero; };
+  for (int r = ty; r < 2 * (kHamTy + 4); r += kHamTy) {   // x halo: zeros, never overwritten
     if (tx == 0) hs4[r * W] = zero;
     if (tx == n4 - 1) hs4[r * W + n4 + 1] = zero;
   }
-  // planes z-2 .. z+3 of this column, the halo row value of plane z (threads ty < 2 and
-  // ty >= kHamTy - 2): every global load is issued one plane ahead of its use
-  const bool halo_lo = ty < 2, halo_hi = ty >= kHamTy - 2;
-  const int yh = halo_lo ? y0 - 2 + ty : y0 + ty + 2;
-  float4 q0 = ld(y, z0 - 2), q1 = ld(y, z0 - 1), q2 = ld(y, z0), q3 = ld(y, z0 + 1), q4 = ld(y, z0 + 2);
-  float4 q5 = ld(y, z0 + 3);
-  float4 hv = (halo_lo || halo_hi) ? ld(yh, z0) : zero;
-  const double sh = shift ? shift[b] : 0.0;
-  const bool act = y < n;
+  float4 q0 = ld(z0 - 2, col), q1 = ld(z0 - 1, col), q2 = ld(z0, col), q3 = ld(z0 + 1, col), q4 = ld(z0 + 2, col);
+  float4 q5 = ld(z0 + 3, col);
+  float4 hv = acth ? ld(z0, colh) : zero;
+  ptrdiff_t v4 = (ptrdiff_t)z0 * nn4 + col;   // this column's point of plane z
+  const float4* V4 = reinterpret_cast<const float4*>(V);
+  const float4* m4 = reinterpret_cast<const float4*>(mask);
+  const float4* j4 = reinterpret_cast<const float4*>(jr) + (HJ ? band : 0);
+  float4* o4 = reinterpret_cast<float4*>(out) + band;
+  float4 vv = zero, m = zero, rr = zero;
+  if (HV) vv = __ldg(V4 + v4);
+  if (HM) m = __ldg(m4 + v4);
+  if (HJ) rr = __ldg(j4 + v4);
+  const float s = shift ? (float)shift[b] : 0.f;
+  const float dj = d0 + s;
+  float4* const own = hs4 + (ty + 2) * W + 1 + tx;
+  float4* const halo = hs4 + (ty < 2 ? ty : ty + 4) * W + 1 + tx;
+  const int np = (kHamTy + 4) * W;
+  int pl = 0;   // this plane's buffer
   for (int z = z0; z < z1; ++z) {
-    const size_t v4 = (size_t)z * nn4 + (size_t)(act ? y : 0) * n4 + tx;
-    float4 vv = zero, m = zero, rr = zero;
-    if (act && V) vv = __ldg(reinterpret_cast<const float4*>(V) + v4);
-    if (act && mask) m = __ldg(reinterpret_cast<const float4*>(mask) + v4);
-    if (act && jr) rr = __ldg(reinterpret_cast<const float4*>(jr) + (size_t)b * N4 + v4);
-    const float4 qn = ld(y, z + 4);
-    const float4 hn = ((halo_lo || halo_hi) && z + 1 < z1) ? ld(yh, z + 1) : zero;
-    __syncthreads();   // the previous plane's neighbour reads are done
-    hs4[(ty + 2) * W + 1 + tx] = q2;
-    if (halo_lo) hs4[ty * W + 1 + tx] = hv;
-    if (halo_hi) hs4[(ty + 4) * W + 1 + tx] = hv;
+    const bool more = z + 1 < z1;
+    float4 qn = zero, hn = zero, vn = zero, mn = zero, rn = zero;
+    if (z + 4 < n) qn = __ldg(f4 + v4 + 4 * (ptrdiff_t)nn4);
+    if (acth && more) hn = __ldg(f4 + v4 + nn4 + (colh - col));
+    if (HV && more) vn = __ldg(V4 + v4 + nn4);
+    if (HM && more) mn = __ldg(m4 + v4 + nn4);
+    if (HJ && more) rn = __ldg(j4 + v4 + nn4);
+    own[pl] = q2;
+    halo[pl] = hv;
     __syncthreads();
-    if (act) {
-      const float4 c = q2;
-      const float4 L = hs4[(ty + 2) * W + tx], R = hs4[(ty + 2) * W + 2 + tx];
-      const float4 ym1 = hs4[(ty + 1) * W + 1 + tx], yp1 = hs4[(ty + 3) * W + 1 + tx];
-      const float4 ym2 = hs4[ty * W + 1 + tx], yp2 = hs4[(ty + 4) * W + 1 + tx];
-      float4 r;
-      r.x = ham_point(c.x, L.z, L.w, c.y, c.z, ym2.x, ym1.x, yp1.x, yp2.x, q0.x, q1.x, q3.x, q4.x, inv12h2);
-      r.y = ham_point(c.y, L.w, c.x, c.z, c.w, ym2.y, ym1.y, yp1.y, yp2.y, q0.y, q1.y, q3.y, q4.y, inv12h2);
-      r.z = ham_point(c.z, c.x, c.y, c.w, R.x, ym2.z, ym1.z, yp1.z, yp2.z, q0.z, q1.z, q3.z, q4.z, inv12h2);
-      r.w = ham_point(c.w, c.y, c.z, R.x, R.y, ym2.w, ym1.w, yp1.w, yp2.w, q0.w, q1.w, q3.w, q4.w, inv12h2);
-      if (V) {
-        r.x += vv.x * c.x;
-        r.y += vv.y * c.y;
-        r.z += vv.z * c.z;
-        r.w += vv.w * c.w;
-      }
-      if (shift) {
-        const float s = (float)sh;
-        r.x += s * c.x;
-        r.y += s * c.y;
-        r.z += s * c.z;
-        r.w += s * c.w;
-      }
-      if (mask) {
-        r.x *= m.x;
-        r.y *= m.y;
-        r.z *= m.z;
-        r.w *= m.w;
-      }
-      if (jr) {
-        const float d = d0 + (float)sh;
-        r.x = c.x + omega * (rr.x - r.x) / d;
-        r.y = c.y + omega * (rr.y - r.y) / d;
-        r.z = c.z + omega * (rr.z - r.z) / d;
-        r.w = c.w + omega * (rr.w - r.w) / d;
-      }
-      reinterpret_cast<float4*>(out)[(size_t)b * N4 + v4] = r;
+    const float4 c = q2;
+    const float4* p = own + pl;
+    const float4 L = p[-1], R = p[1], ym1 = p[-W], yp1 = p[W], ym2 = p[-2 * W], yp2 = p[2 * W];
+    float4 r;
+    r.x = ham_point(c.x, L.z, L.w, c.y, c.z, ym2.x, ym1.x, yp1.x, yp2.x, q0.x, q1.x, q3.x, q4.x, inv12h2);
+    r.y = ham_point(c.y, L.w, c.x, c.z, c.w, ym2.y, ym1.y, yp1.y, yp2.y, q0.y, q1.y, q3.y, q4.y, inv12h2);
+    r.z = ham_point(c.z, c.x, c.y, c.w, R.x, ym2.z, ym1.z, yp1.z, yp2.z, q0.z, q1.z, q3.z, q4.z, inv12h2);
+    r.w = ham_point(c.w, c.y, c.z, R.x, R.y, ym2.w, ym1.w, yp1.w, yp2.w, q0.w, q1.w, q3.w, q4.w, inv12h2);
+    if (HV) {
+      r.x += vv.x * c.x;
+      r.y += vv.y * c.y;
+      r.z += vv.z * c.z;
+      r.w += vv.w * c.w;
     }
+    if (shift) {
+      r.x += s * c.x;
+      r.y += s * c.y;
+      r.z += s * c.z;
+      r.w += s * c.w;
+    }
+    if (HM) {
+      r.x *= m.x;
+      r.y *= m.y;
+      r.z *= m.z;
+      r.w *= m.w;
+    }
+    if (HJ) {
+      r.x = c.x + omega * (rr.x - r.x) / dj;
+      r.y = c.y + omega * (rr.y - r.y) / dj;
+      r.z = c.z + omega * (rr.z - r.z) / dj;
+      r.w = c.w + omega * (rr.w - r.w) / dj;
+    }
+    o4[v4] = r;
     q0 = q1;
     q1 = q2;
     q2 = q3;
@@ -190,6 +204,11 @@ __global__ void __launch_bounds__(512) k_ham_apply_z(const float* __restrict__ f
     q4 = q5;
     q5 = qn;
     hv = hn;
+    vv = vn;
+    m = mn;
+    rr = rn;
+    v4 += nn4;
+    pl = np - pl;
   }
 }
 
@@ -205,15 +224,19 @@ dim3 ham_grid(int nb, int n) {
 
 bool ham_tiles_ok(const float* f, int n, const float* V, const float* mask, const float* out, const float* jr) {
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  return n % 4 == 0 && (n / 4) * kHamTy <= 512 && al16(f) && al16(out) && (!V || al16(V)) && (!mask || al16(mask)) &&
+  return n % 4 == 0 && n <= 256 && al16(f) && al16(out) && (!V || al16(V)) && (!mask || al16(mask)) &&
          (!jr || al16(jr));
 }
+// jr: a Jacobi sweep, which takes V = 0
 void launch_ham_tiles(const float* f, int nb, int n, float inv12h2, const float* V, const double* shift,
                       const float* mask, const float* jr, float d0, float omega, float* out, cudaStream_t s) {
   const int n4 = n / 4;
-  const dim3 grid((n + kHamTy - 1) / kHamTy, (n + kHamZc - 1) / kHamZc, nb), block(n4, kHamTy);
-  const size_t smem = sizeof(float4) * (size_t)(kHamTy + 4) * (n4 + 2);
-  k_ham_apply_z<<<grid, block, smem, s>>>(f, n, inv12h2, V, shift, mask, jr, d0, omega, out);
+  const dim3 grid(n / kHamTy, (n + kHamZc - 1) / kHamZc, nb), block(n4, kHamTy);
+  const size_t smem = 2 * sizeof(float4) * (size_t)(kHamTy + 4) * (n4 + 2);
+  auto kern = jr ? (mask ? k_ham_apply_z<false, true, true> : k_ham_apply_z<false, false, true>)
+              : V ? (mask ? k_ham_apply_z<true, true, false> : k_ham_apply_z<true, false, false>)
+                  : (mask ? k_ham_apply_z<false, true, false> : k_ham_apply_z<false, false, false>);
+  kern<<<grid, block, smem, s>>>(f, n, inv12h2, V, shift, mask, jr, d0, omega, out);
 }
 
 // out = H f over nb bands: the z-marching tiles where the layout allows, else one thread
@@ -296,16 +319,23 @@ __global__ void k_residual(const float* __restrict__ psi, const float* __restric
 }
 
 // one damped-Jacobi sweep for (K + T) x = r:  x_out = x_in + omega (r - (K + T) x_in) / d,
-// d = 3.75 / h^2 + T; with x_in null the sweep starts from x0 = r / d.
+// d = 3.75 / h^2 + T; with x_in null the sweep starts from x0 = r / d.  A row per blockIdx.y.
+// The start alone (the tiled path's only use) takes four points of a row per access.
 __global__ void k_ke_jacobi(const float* __restrict__ r, const float* __restrict__ xin, const float* __restrict__ axin,
-                            const double* __restrict__ T, int nb, size_t N, float d0, float omega,
-                            float* __restrict__ xout) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)nb * N;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const size_t b = i / N;
-    const float d = d0 + (float)T[b];
-    xout[i] = xin ? xin[i] + omega * (r[i] - axin[i]) / d : r[i] / d;
+                            const double* __restrict__ T, size_t N, float d0, float omega, float* __restrict__ xout) {
+  const size_t row = (size_t)blockIdx.y * N, stride = (size_t)gridDim.x * blockDim.x;
+  const float d = d0 + (float)T[blockIdx.y];
+  if (!xin && (N & 3) == 0 && aligned16(r) && aligned16(xout)) {
+    const float4* r4 = reinterpret_cast<const float4*>(r + row);
+    float4* x4 = reinterpret_cast<float4*>(xout + row);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N / 4; i += stride) {
+      const float4 v = r4[i];
+      x4[i] = make_float4(v.x / d, v.y / d, v.z / d, v.w / d);
+    }
+    return;
   }
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N; i += stride)
+    xout[row + i] = xin ? xin[row + i] + omega * (r[row + i] - axin[row + i]) / d : r[row + i] / d;
 }
 
 // T_i = max(theta_i - <psi_i, V psi_i>, 0): the orbital's kinetic energy
@@ -1134,18 +1164,18 @@ int rsx_eig_step(rsx_eig* e, rsx_net* net, int jacobi_sweeps, double* theta_host
     // that the last sweep writes W
     float* buf[2] = {wp, e->tmp + k * N};
     int cur = jacobi_sweeps % 2;
-    k_ke_jacobi<<<(unsigned)blocks_for(k * N), 256, 0, s>>>(e->R, nullptr, nullptr, T, k, N, d0, omega, buf[cur]);
+    k_ke_jacobi<<<dim3((unsigned)row_blocks(N, k), k), 256, 0, s>>>(e->R, nullptr, nullptr, T, N, d0, omega, buf[cur]);
     for (int sw = 0; sw < jacobi_sweeps; ++sw, cur ^= 1)
       launch_ham_tiles(buf[cur], k, e->n, (float)(1.0 / (12.0 * e->h * e->h)), nullptr, T, e->mask, e->R, d0, omega,
                        buf[cur ^ 1], s);
     rc = ecuda(e, cudaGetLastError(), "jacobi sweeps");
     if (rc) return rc;
   } else {
-    k_ke_jacobi<<<(unsigned)blocks_for(k * N), 256, 0, s>>>(e->R, nullptr, nullptr, T, k, N, d0, omega, x);
+    k_ke_jacobi<<<dim3((unsigned)row_blocks(N, k), k), 256, 0, s>>>(e->R, nullptr, nullptr, T, N, d0, omega, x);
     for (int sw = 0; sw < jacobi_sweeps; ++sw) {
       rc = ham(e, x, k, ax, T, nullptr, s);
       if (rc) return rc;
-      k_ke_jacobi<<<(unsigned)blocks_for(k * N), 256, 0, s>>>(e->R, x, ax, T, k, N, d0, omega, e->tmp + k * N);
+      k_ke_jacobi<<<dim3((unsigned)row_blocks(N, k), k), 256, 0, s>>>(e->R, x, ax, T, N, d0, omega, e->tmp + k * N);
       rc = ecuda(e, cudaMemcpyAsync(x, e->tmp + k * N, k * N * sizeof(float), cudaMemcpyDeviceToDevice, s), "jacobi copy");
       if (rc) return rc;
     }
