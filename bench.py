@@ -239,9 +239,9 @@ def algorithmic_flops(kernel, shape, nq, npsi_out):
                  + nz * lf(Ay, "inv_keep_half"))
         return nq * Hx * plane
     if kernel == "pass1_x_forward":
-        return nq * nz * (ny // 2) * (line_flops(Ax, "fwd_pruned") + 8 * Hx)
+        return nq * nz * (ny // 2) * (line_flops_l8(Ax, "fwd_pruned") + 8 * Hx)
     if kernel == "pass3_x_inverse_accumulate":
-        return nq * nz * (ny // 2) * (line_flops(Ax, "inv_keep_half") + 2 * 16 * Ax + 4 * nx)
+        return nq * nz * (ny // 2) * (line_flops_l8(Ax, "inv_keep_half") + 2 * 16 * Ax + 4 * nx)
     return None
 
 
