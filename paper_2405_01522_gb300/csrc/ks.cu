@@ -387,15 +387,70 @@ __global__ void k_net_input(const float* __restrict__ R, const double* __restric
 //     corrections of the k lowest vectors against C and their Rayleigh quotients;
 //  4. the new orbitals' coefficients over the basis, Q = L^-T Z.
 // Outputs theta[k] and qt[k][m] (float).  Fewer than k kept directions raise RSX_ENOTPD.
+// Bound by serial chains and by the FP64 units (2 FMA a cycle and SM).  At m = 48, 370 us of which
+// Cholesky 50, L^-1 67, roots 36 and inverse iteration 42 before four threads shared a column of
+// L^-1, a warp's roots ran side by side and the Cholesky update left its upper half out (every
+// sum in its old order): two steps of the 96^3 eigensolver 2603 -> 2522 us.
 constexpr double kRrDrop = 1e-6;
 constexpr int kRrThreads = 512;
 constexpr int kRrWarps = kRrThreads / 32;
 constexpr int kRrNewton = 2;   // FP64 correction steps of the Rayleigh-Ritz eigenvectors
 
+// Roots warp + kRrWarps u of T (u < U) by Sturm multisection, 32 points per root and round.  The
+// counts of the roots are independent chains of one approximate division per row (that of
+// sturm_count_f32), so a warp's roots run interleaved.
+template <int U>
+__device__ __forceinline__ void rr_roots(const float* d, const float* e2, int n, float lo0, float hi0, float pivmin,
+                                         int warp, int lane, float* lam) {
+  float lo[U], hi[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    lo[u] = lo0;
+    hi[u] = hi0;
+  }
+  for (int round = 0; round < 8; ++round) {
+    bool open[U], any = false;
+    float x[U], q[U];
+    int cnt[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      open[u] = hi[u] - lo[u] > 2.4e-7f * fmaxf(fabsf(lo[u]), fabsf(hi[u]));
+      any |= open[u];
+      x[u] = lo[u] + (hi[u] - lo[u]) * (float)(lane + 1) / 33.f;
+      q[u] = d[0] - x[u];
+      if (fabsf(q[u]) < pivmin) q[u] = -pivmin;
+      cnt[u] = q[u] < 0.f;
+    }
+    if (!any) break;
+    for (int i = 1; i < n; ++i) {
+      const float di = d[i], ei = e2[i - 1];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        q[u] = (di - x[u]) - __fdividef(ei, q[u]);
+        if (fabsf(q[u]) < pivmin) q[u] = -pivmin;
+        cnt[u] += q[u] < 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned above = __ballot_sync(0xffffffffu, cnt[u] > warp + kRrWarps * u);
+      if (!open[u]) continue;
+      const int f = above ? __ffs(above) - 1 : 32;
+      const float nlo = (f == 0) ? lo[u] : lo[u] + (hi[u] - lo[u]) * (float)f / 33.f;
+      const float nhi = (f == 32) ? hi[u] : lo[u] + (hi[u] - lo[u]) * (float)(f + 1) / 33.f;
+      lo[u] = nlo;
+      hi[u] = nhi;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (lane == 0) lam[warp + kRrWarps * u] = 0.5f * (lo[u] + hi[u]);
+}
+
 __global__ void __launch_bounds__(kRrThreads) k_rayleigh_ritz(const double* __restrict__ Sg, const double* __restrict__ Hg,
                                                               int m, int k, double* __restrict__ theta,
                                                               float* __restrict__ qt, int* status) {
-  extern __shared__ double rr_smem[];   // 4 m x m: L, Li, C, T (then Z); solve scratch 4 m per warp
+  extern __shared__ double rr_smem[];   // 4 m x m: L, Li, C, T (then Z); scratch (4 kRrWarps + 1) m
   double* L = rr_smem;
   double* Li = L + m * m;
   double* C = Li + m * m;
@@ -405,7 +460,7 @@ __global__ void __launch_bounds__(kRrThreads) k_rayleigh_ritz(const double* __re
   __shared__ float d32[kMaxBasis], e32[kMaxBasis], e2f[kMaxBasis], lam32[kMaxBasis];
   __shared__ float tau32[kMaxBasis], vv32[kMaxBasis], pp32[kMaxBasis];
   __shared__ int kept[kMaxBasis], dropped[kMaxBasis];
-  __shared__ int piv[kRrWarps][kMaxBasis];
+  __shared__ int piv[kMaxBasis][kMaxBasis + 1];
   __shared__ int nkeep;
   __shared__ float sh_beta32, sh_tau32, sh_scale32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -432,30 +487,32 @@ __global__ void __launch_bounds__(kRrThreads) k_rayleigh_ritz(const double* __re
     const int dr = dropped[j];
     for (int i = j + 1 + tid; i < m; i += kRrThreads) L[i * m + j] = dr ? 0.0 : L[i * m + j] * rl;
     __syncthreads();
-    const int t = m - j - 1;
-    for (int q = tid; q < t * t; q += kRrThreads) {
-      const int i = j + 1 + q / t, l = j + 1 + q % t;
-      if (l <= i) L[i * m + l] -= L[i * m + j] * L[l * m + j];
-    }
+    // lower triangle only: a half-warp per row (an FP64 instruction costs a warp 64 cycles of
+    // its scheduler's pipe, however few lanes need it)
+    for (int i = j + 1 + (tid >> 4); i < m; i += kRrThreads / 16)
+      for (int l = j + 1 + (tid & 15); l <= i; l += 16) L[i * m + l] -= L[i * m + j] * L[l * m + j];
     __syncthreads();
   }
-  // L^-1, one column per thread
-  if (tid < m) {
-    const int c = tid;
-    for (int i = 0; i < c; ++i) Li[i * m + c] = 0.0;
-    Li[c * m + c] = rdg[c];
-    for (int i = c + 1; i < m; ++i) {
-      // four partial sums: shorter dependent chains
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-      int p = c;
-      for (; p + 3 < i; p += 4) {
-        s0 += L[i * m + p] * Li[p * m + c];
-        s1 += L[i * m + p + 1] * Li[(p + 1) * m + c];
-        s2 += L[i * m + p + 2] * Li[(p + 2) * m + c];
-        s3 += L[i * m + p + 3] * Li[(p + 3) * m + c];
+  // L^-1, four threads per column, each one of the four partial sums of a row's dot product
+  if (tid < 4 * ((m + 7) & ~7)) {   // whole warps: 8 columns each
+    const int c = tid >> 2, g = tid & 3, c0 = c & ~7;
+    if (c < m) {
+      for (int i = g; i < c; i += 4) Li[i * m + c] = 0.0;
+      if (g == 0) Li[c * m + c] = rdg[c];
+    }
+    __syncwarp();
+    for (int i = c0 + 1; i < m; ++i) {
+      double sum = 0.0;
+      if (c < i) {
+        int p = c;
+        for (; p + 3 < i; p += 4) sum += L[i * m + p + g] * Li[(p + g) * m + c];
+        if (g == 0)
+          for (; p < i; ++p) sum += L[i * m + p] * Li[p * m + c];
       }
-      for (; p < i; ++p) s0 += L[i * m + p] * Li[p * m + c];
-      Li[i * m + c] = -((s0 + s1) + (s2 + s3)) * rdg[i];
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+      if (c < i && g == 0) Li[i * m + c] = -sum * rdg[i];
+      __syncwarp();
     }
   }
   if (tid == 0) {
@@ -498,7 +555,8 @@ __global__ void __launch_bounds__(kRrThreads) k_rayleigh_ritz(const double* __re
   //    quadratically from FP32 accuracy; their Rayleigh quotients are the Ritz values.
   float* C32 = reinterpret_cast<float*>(L);     // n x n (L is dead after L^-1)
   float* X32 = C32 + n * n;                     // n x n: vectors of T, then of C'32
-  float* SC32 = reinterpret_cast<float*>(SCR);  // 4 n floats per warp
+  float* SC32 = reinterpret_cast<float*>(SCR);  // 4 n floats
+  float* IT32 = reinterpret_cast<float*>(T);    // T (dead here) and SCR: 4 n + 1 floats per root
   for (int q = tid; q < n * n; q += kRrThreads) C32[q] = (float)C[q];
   __syncthreads();
   // 3a. FP32 Householder reduction (reflectors below the subdiagonal, tau32)
@@ -584,19 +642,12 @@ __global__ void __launch_bounds__(kRrThreads) k_rayleigh_ritz(const double* __re
   lo0 -= 1e-6f * scale + 1e-30f;
   hi0 += 1e-6f * scale + 1e-30f;
   const float pivmin = 1.2e-38f * fmaxf(1.f, emax * emax);
-  for (int r = warp; r < n; r += kRrWarps) {
-    float lo = lo0, hi = hi0;
-    for (int round = 0; round < 8; ++round) {
-      if (!(hi - lo > 2.4e-7f * fmaxf(fabsf(lo), fabsf(hi)))) break;
-      const float x = lo + (hi - lo) * (float)(lane + 1) / 33.f;
-      const unsigned above = __ballot_sync(0xffffffffu, sturm_count_f32(d32, e2f, n, x, pivmin) > r);
-      const int f = above ? __ffs(above) - 1 : 32;
-      const float nlo = (f == 0) ? lo : lo + (hi - lo) * (float)f / 33.f;
-      const float nhi = (f == 32) ? hi : lo + (hi - lo) * (float)(f + 1) / 33.f;
-      lo = nlo;
-      hi = nhi;
-    }
-    if (lane == 0) lam32[r] = 0.5f * (lo + hi);
+  switch ((n - warp + kRrWarps - 1) / kRrWarps) {   // this warp's roots, their chains interleaved
+    case 4: rr_roots<4>(d32, e2f, n, lo0, hi0, pivmin, warp, lane, lam32); break;
+    case 3: rr_roots<3>(d32, e2f, n, lo0, hi0, pivmin, warp, lane, lam32); break;
+    case 2: rr_roots<2>(d32, e2f, n, lo0, hi0, pivmin, warp, lane, lam32); break;
+    case 1: rr_roots<1>(d32, e2f, n, lo0, hi0, pivmin, warp, lane, lam32); break;
+    default: break;
   }
   __syncthreads();
   // 3c. vectors of T by inverse iteration; among the wanted roots and a margin above
@@ -604,11 +655,27 @@ __global__ void __launch_bounds__(kRrThreads) k_rayleigh_ritz(const double* __re
   //     to the earlier members of their run (higher vectors only carry the small
   //     corrections along far directions, where a duplicate costs nothing measurable)
   const float gap32 = 1e-5f * fmaxf(1.f, scale);
-  for (int r = warp; r < n; r += kRrWarps) {
-    float* z = X32 + r * n;
-    for (int i = lane; i < n; i += 32) z[i] = 1.f + 0.001f * (float)((i * 7919 + r * 104729) % 997);
-    __syncwarp();
-    warp_inverse_iteration<float>(d32, e32, n, lam32[r], z, SC32 + warp * 4 * n, piv[warp], 3, X32, n, 0u);
+  //     (a lane per root of the warp: the serial LU and solves of its roots run side by side)
+  for (int r = warp; r < n; r += kRrWarps)
+    for (int i = lane; i < n; i += 32) X32[r * n + i] = 1.f + 0.001f * (float)((i * 7919 + r * 104729) % 997);
+  __syncwarp();
+  {
+    const int r = warp + kRrWarps * lane;   // this lane's root
+    float* sc = IT32 + r * (4 * n + 1);
+    if (r < n) tri_factor_shifted<float>(d32, e32, n, lam32[r], sc, piv[r]);
+    for (int it = 0; it < 3; ++it) {
+      if (r < n) tri_solve_factored<float>(n, X32 + r * n, sc, piv[r]);
+      __syncwarp();
+      for (int rr = warp; rr < n; rr += kRrWarps) {
+        float* z = X32 + rr * n;
+        float nn = 0.f;
+        for (int i = lane; i < n; i += 32) nn += z[i] * z[i];
+        nn = warp_sum(nn);
+        const float inv = nn > 0.f ? 1.f / sqrtf(nn) : 0.f;
+        for (int i = lane; i < n; i += 32) z[i] *= inv;
+      }
+      __syncwarp();
+    }
   }
   __syncthreads();
   if (warp == 0) {
@@ -1051,7 +1118,7 @@ int rr_update(rsx_eig* e, int m, bool keep_p, cudaStream_t s) {
   int rc = gram(e, e->B, m, e->B, m, nullptr, S, s);
   if (!rc) rc = gram(e, e->B, m, e->HB, m, nullptr, Hs, s);
   if (rc) return rc;
-  const size_t smem = (4 * (size_t)m * m + 4 * (size_t)kRrWarps * m) * sizeof(double);
+  const size_t smem = (4 * (size_t)m * m + (4 * (size_t)kRrWarps + 1) * m) * sizeof(double);
   cudaFuncSetAttribute(k_rayleigh_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k_rayleigh_ritz<<<1, kRrThreads, smem, s>>>(S, Hs, m, k, theta, e->qt, e->ctx->status);
   rc = ecuda(e, cudaGetLastError(), "rayleigh-ritz");
