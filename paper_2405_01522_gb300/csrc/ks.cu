@@ -258,7 +258,8 @@ __global__ void k_mask_rows(float* __restrict__ X, const float* __restrict__ mas
 }
 
 // part[b * gridDim.x + blk] = this block's share of sum_v X_b(v) Y_b(v) (w(v)) for row
-// b = blockIdx.y (FP32 products of four points, FP64 sums).  N % 4 == 0, rows 16-byte aligned.
+// b = blockIdx.y (FP32 products of four points, FP64 sums); point by point where N % 4 != 0 (an
+// odd edge: rows beyond the first are not 16-byte aligned) or an array is not aligned.
 __global__ void k_row_dots(const float* __restrict__ X, const float* __restrict__ Y, const float* __restrict__ w,
                            size_t N, double* __restrict__ part) {
   __shared__ double red[32];
@@ -267,7 +268,14 @@ __global__ void k_row_dots(const float* __restrict__ X, const float* __restrict_
   const float4* y4 = reinterpret_cast<const float4*>(Y + (size_t)b * N);
   const float4* w4 = reinterpret_cast<const float4*>(w);
   double acc = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N / 4; i += (size_t)gridDim.x * blockDim.x) {
+  const bool vec = (N & 3) == 0 && aligned16(X) && aligned16(Y) && aligned16(w);
+  if (!vec) {
+    const float* x = X + (size_t)b * N;
+    const float* y = Y + (size_t)b * N;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x)
+      acc += (double)(x[i] * y[i] * (w ? w[i] : 1.f));
+  }
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; vec && i < N / 4; i += (size_t)gridDim.x * blockDim.x) {
     const float4 a = x4[i], c = y4[i];
     float4 p = make_float4(a.x * c.x, a.y * c.y, a.z * c.z, a.w * c.w);
     if (w) {
