@@ -246,14 +246,14 @@ __global__ void __launch_bounds__(cv_threads(IN), 2) k_conv(const __grid_constan
       bulk_load(wsm, a.wimg, kW, &wbar);
     }
     __syncwarp();
-    bool ok = __all_sync(0xffffffffu, mbar_wait(&wbar, 0, abort_flag));
+    bool ok = mbar_wait_warp(&wbar, 0, abort_flag);
     const uint64_t a_desc = smem_desc(smem_u32(slots), 2 * kCvHX * 16, 4 * kCvHX * 16);
     const uint64_t b_desc = smem_desc(smem_u32(wsm), 128, 256);
     int n = 0, p = 0;
     for (; ok && p < np; ++p) {
       if (plane_in(p)) {
         const int slot = n % kCvSlots;
-        ok = __all_sync(0xffffffffu, mbar_wait(&full[slot], (uint32_t)((n / kCvSlots) & 1), abort_flag));
+        ok = mbar_wait_warp(&full[slot], (uint32_t)((n / kCvSlots) & 1), abort_flag);
         if (!ok) break;
         // slices p - 2 + k, k = k0 .. k1 of this plane
         const int k0 = max(0, 2 - p), nk = min(2, nzl - 1 - (p - 2)) - k0 + 1;
@@ -346,8 +346,7 @@ __global__ void __launch_bounds__(cv_threads(IN), 2) k_conv(const __grid_constan
       bsum[c] = 0.f;
     }
     for (int s = 0; s < nzl; ++s) {
-      if (!mbar_wait(&ready[s + 2], 0, abort_flag)) break;
-      __syncwarp();
+      if (!mbar_wait_warp(&ready[s + 2], 0, abort_flag)) break;   // lanes outside the box vote too
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float acc[16];
       tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(16 * s), acc);
@@ -536,9 +535,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad(const __grid_constant__
     int k = 0;
     for (; k < nz; ++k) {
       for (; ok && loaded < k + 3; ++loaded)
-        ok = __all_sync(0xffffffffu, mbar_wait(&fin[loaded % kWgInSlots], (uint32_t)((loaded / kWgInSlots) & 1), abort_flag));
+        ok = mbar_wait_warp(&fin[loaded % kWgInSlots], (uint32_t)((loaded / kWgInSlots) & 1), abort_flag);
       const int gslot = k % kWgGSlots;
-      if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&fg[gslot], (uint32_t)((k / kWgGSlots) & 1), abort_flag));
+      if (ok) ok = mbar_wait_warp(&fg[gslot], (uint32_t)((k / kWgGSlots) & 1), abort_flag);
       if (!ok) break;
       const uint64_t bh = b_desc + (uint64_t)(gslot * (kWgG / 16)), bl = bh + kWgX;
 #pragma unroll
