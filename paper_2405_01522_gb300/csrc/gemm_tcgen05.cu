@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     bool ok = true;
     for (int ch = 0; ch < nchunk; ++ch) {
       const int b = ch & 1, use = ch >> 1;
-      ok = mbar_wait(&tfull_bar[b], (uint32_t)(use & 1), abort_flag);
+      ok = mbar_wait_warp(&tfull_bar[b], (uint32_t)(use & 1), abort_flag);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * kBN + cg * 32);
