@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(kGsThreads, 2) k_gram_stream(const float* __re
   for (int o = 0; o < 16; ++o) ah[o] = al[o] = 0.f;
   bool ok = true;
   for (long long i = 0; i < mine; ++i) {
-    ok = tc::mbar_wait(&full[i % STAGES], (uint32_t)((i / STAGES) & 1), &abort_flag);
+    ok = tc::mbar_wait_warp(&full[i % STAGES], (uint32_t)((i / STAGES) & 1), &abort_flag);
     if (!ok) break;
     const size_t r0 = (cb + (size_t)i * ncb) * CHUNK;
     const int q4 = (int)min((size_t)CHUNK, N - r0) >> 2;

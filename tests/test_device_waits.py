@@ -39,7 +39,7 @@ def enclosing_loop(text, pos):
     return ""
 
 
-@pytest.mark.parametrize("name", ["convnet.cu", "gemm_tcgen05.cu"])
+@pytest.mark.parametrize("name", ["convnet.cu", "gemm_tcgen05.cu", "dense.cu"])
 def test_waits_beside_warp_collectives_are_the_warps(name):
     text = source(name)
     calls = [m.start() for m in re.finditer(r"\bmbar_wait\(", text)]
