@@ -273,8 +273,11 @@ __global__ void __launch_bounds__(cv_threads(IN), 2) k_conv(const __grid_constan
       }
       if (lead) mma_commit(&ready[p]);
     }
-    // no arrival may land after the CTA exits: the last commit of every barrier (bounded waits)
-    const int last = ok ? np - 1 : (n > 0 ? (p < np ? p : np - 1) : -1);
+    // no copy or arrival may land after the CTA exits: the weights, then the last commit of every
+    // barrier (bounded waits; after a time-out at plane p, ready[p] closes what came before it)
+    for (uint32_t k = 0; k < kWaitLimit && !mbar_try_wait(&wbar, 0); ++k) {
+    }
+    const int last = ok ? np - 1 : (p > 0 ? p : -1);
     if (!ok && last >= 0 && lead) mma_commit(&ready[last]);
     for (int i = max(0, n - kCvSlots); i < n; ++i)
       for (uint32_t k = 0; k < kWaitLimit && !mbar_try_wait(&empty[i % kCvSlots], (uint32_t)((i / kCvSlots) & 1)); ++k) {

@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     if (lane == 0) {
       // ---------------- MMA issuer: chunks of kChunk K blocks into alternating TMEM buffers
       bool live = true;
+      int done = 0, last = -1;   // K blocks whose stage, and last chunk whose accumulator, was committed
       for (int ch = 0; ch < nchunk && live; ++ch) {
         const int b = ch & 1, use = ch >> 1;
         if (use > 0 && !mbar_wait(&tempty_bar[b], (uint32_t)((use - 1) & 1), abort_flag)) break;
@@ -197,8 +198,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             mma_bf16(acc, dl_i + adv, dh_j + adv, 1u);
           }
           mma_commit(&empty_bar[s]);
+          done = it + 1;
         }
         mma_commit(&tfull_bar[b]);   // fires when this chunk's MMAs have completed
+        last = ch;
+      }
+      // no arrival may land after the CTA exits, nor its TMEM be freed under an MMA (bounded waits)
+      for (int it = done > kStages ? done - kStages : 0; it < done; ++it)
+        for (uint32_t i = 0; i < kWaitLimit && !mbar_try_wait(&empty_bar[it % kStages], (uint32_t)((it / kStages) & 1)); ++i) {
+        }
+      for (uint32_t i = 0; last >= 0 && i < kWaitLimit && !mbar_try_wait(&tfull_bar[last & 1], (uint32_t)((last >> 1) & 1)); ++i) {
       }
     }
   } else {

@@ -3,7 +3,9 @@ tensor memory or have copies in flight.
 
 * In a loop that contains warp-collective instructions the wait is the warp's, mbar_wait_warp: with
   mbar_wait the lanes decide one by one, and after a time-out those that stay would run
-  collectives without those that left."""
+  collectives without those that left.
+* Every mbarrier that copies or MMA completions arrive on is waited for once more, with a limit,
+  before the CTA leaves (mbar_try_wait): nothing may land in its shared memory afterwards."""
 import os
 import re
 
@@ -48,3 +50,18 @@ def test_waits_beside_warp_collectives_are_the_warps(name):
     for pos in calls:
         body = enclosing_loop(text, pos)
         assert not COLLECTIVE.search(body), f"{name}: per-lane wait in a loop with warp collectives:\n{body[:400]}"
+
+
+@pytest.mark.parametrize("name", ["convnet.cu", "gemm_tcgen05.cu"])
+def test_barriers_of_asynchronous_arrivals_are_drained(name):
+    text = source(name)
+    arriving = set(re.findall(r"\bmma_commit\(&(\w+)", text))
+    for call in re.findall(r"\b(?:tma_load_\dd|bulk_load)\(([^;]*);", text):
+        arriving |= set(re.findall(r"&(\w+)", call))
+    barriers = set()
+    for decl in re.findall(r"__shared__ __align__\(8\) uint64_t ([^;]*);", text):
+        barriers |= set(re.findall(r"(\w+)(?:\[[^\]]*\])?(?:,|$)", decl))
+    arriving &= barriers
+    assert len(arriving) >= 3
+    drained = set(re.findall(r"\bmbar_try_wait\(&(\w+)", text))
+    assert arriving <= drained, f"{name}: not drained: {sorted(arriving - drained)}"
