@@ -22,8 +22,34 @@ namespace rsx {
 // while the kernel before it in the stream drains.  Every pass starts with pdl_wait(), before
 // its first access to memory that kernel touches (it returns when that kernel is complete
 // and its writes are visible), and lets its own successor be set up from its start.
+// What the kernel before may still be writing at that time -- the orbitals, the intermediate -- must
+// not be read through __ldg or const __restrict__ pointers: those make ld.global.nc, whose data
+// may not change while the kernel runs and which the wait's memory clobber does not hold
+// back.  It is read by ld_dep, or by plain loads through unqualified pointers.  The tables written by
+// rsx_create are constant.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// coherent global loads, in program order with pdl_wait (volatile)
+__device__ __forceinline__ float ld_dep(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_dep(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_dep(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 ld_dep(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
 
 __host__ __device__ constexpr int line_tw_count(int A, int neg) { return neg - 1 > 2 * A - neg ? neg - 1 : 2 * A - neg; }
 __host__ __device__ constexpr int line_neg(int A) {   // 2A: no negative rows

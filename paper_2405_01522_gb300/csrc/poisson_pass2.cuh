@@ -77,7 +77,7 @@ __device__ __forceinline__ void p2_scale4(Cx<float>* u, float4 m) {
 // Shared memory: [line scratch] [plane NB x p2_pitch].
 template <typename R, int A, bool DSMEM>
 __global__ void __launch_bounds__(p2_threads<R>(A), p2_min_ctas<R>(A))
-    k_pass2(Geom g, int nq, Cx<R>* __restrict__ inter, const Cx<R>* __restrict__ twg, const R* __restrict__ vl,
+    k_pass2(Geom g, int nq, Cx<R>* inter, const Cx<R>* __restrict__ twg, const R* __restrict__ vl,
             Cx<R>* gscratch) {
   using S = typename P2Split<R, A>::type;
   constexpr int NL = p2_lines<R>(A), LN = S::LANES, NIN = S::NIN;

@@ -53,12 +53,12 @@ struct Vec16<double> {
 
 // two consecutive complex values from / to global memory
 __device__ __forceinline__ void ld_pair(const Cx<float>* p, Cx<float>& a, Cx<float>& b) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
+  const float4 v = ld_dep(reinterpret_cast<const float4*>(p));
   a = cx<float>(v.x, v.y);
   b = cx<float>(v.z, v.w);
 }
 __device__ __forceinline__ void ld_pair(const Cx<double>* p, Cx<double>& a, Cx<double>& b) {
-  const double2 v = reinterpret_cast<const double2*>(p)[0], w = reinterpret_cast<const double2*>(p)[1];
+  const double2 v = ld_dep(reinterpret_cast<const double2*>(p)), w = ld_dep(reinterpret_cast<const double2*>(p) + 1);
   a = cx<double>(v.x, v.y);
   b = cx<double>(w.x, w.y);
 }
@@ -81,7 +81,7 @@ __device__ __forceinline__ void st_pair(Cx<double>* p, Cx<double> a, Cx<double> 
 // the pairs are the fastest index in groups of G, so that the CTAs in flight share their rows
 // and the orbital rows they multiply are read from HBM once per group and then hit in L2.
 template <typename R, int A>
-__global__ void __launch_bounds__(32 * kXWarps, p1_min_ctas<R>(A)) k_pass1(Geom g, PairMap<R> pm, int q0, int nq, Cx<R>* __restrict__ inter,
+__global__ void __launch_bounds__(32 * kXWarps, p1_min_ctas<R>(A)) k_pass1(Geom g, PairMap<R> pm, int q0, int nq, Cx<R>* inter,
                                                        const Cx<R>* __restrict__ twx) {
   using X = XWarp<R, A>;
   using S = typename X::S;
@@ -119,8 +119,8 @@ __global__ void __launch_bounds__(32 * kXWarps, p1_min_ctas<R>(A)) k_pass1(Geom 
 #pragma unroll
     for (int i = 0; i < IT; ++i)
       if (NV % 32 == 0 || lane + 32 * i < NV) {
-        a[i] = __ldg(reinterpret_cast<const typename V::T*>(f1) + lane + 32 * i);
-        c[i] = __ldg(reinterpret_cast<const typename V::T*>(f2) + lane + 32 * i);
+        a[i] = ld_dep(reinterpret_cast<const typename V::T*>(f1) + lane + 32 * i);
+        c[i] = ld_dep(reinterpret_cast<const typename V::T*>(f2) + lane + 32 * i);
       }
 #pragma unroll
     for (int i = 0; i < IT; ++i)
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(32 * kXWarps, p1_min_ctas<R>(A)) k_pass1(Geom 
   } else {   // orbitals off 16-byte boundaries
     for (int e = lane; e < 8 * NB; e += 32) {
       const int r = e / NB, x = e - r * NB;
-      tile[r * RP + x] = R(0.5) * (__ldg(f1 + e) * __ldg(f2 + e));
+      tile[r * RP + x] = R(0.5) * (ld_dep(f1 + e) * ld_dep(f2 + e));
     }
   }
   __syncwarp();
@@ -177,8 +177,7 @@ __global__ void __launch_bounds__(32 * kXWarps, p1_min_ctas<R>(A)) k_pass1(Geom 
 // the transform that hides them).  The accumulators stay in registers over the entries.
 template <typename R, int A>
 __global__ void __launch_bounds__(32 * kXWarps, p3_min_ctas<R>(A)) k_pass3(Geom g, PairMap<R> pm, int q0, int p0, int np, int pot,
-                                                       const Cx<R>* __restrict__ inter,
-                                                       const Cx<R>* __restrict__ twx, R* __restrict__ out) {
+                                                       const Cx<R>* inter, const Cx<R>* __restrict__ twx, R* out) {
   using X = XWarp<R, A>;
   using S = typename X::S;
   constexpr int NB = X::NB, RP = X::RP, E = 16 / (int)sizeof(R), J = Line<A>::J, A2 = 2 * A;
