@@ -392,12 +392,14 @@ const char* rsx_kernel_name(int kernel);
 
 /* Failure detection, exercised without faulting the GPU (testing aids; the paper has no
  * counterpart).
- * rsx_set_wait_limit: spin rounds a CTA of the context's cooperative kernels (the
- *   grid-wide barrier of the multi-CTA Householder reduction) waits before giving up;
- *   spins < 0 restores the default (2^24 rounds, far beyond any normal wait), 0 makes
- *   every CTA but the last arriver give up at once.  A CTA that gives up marks the
- *   barrier aborted, every CTA leaves at its next barrier, and rsx_sync_status reports
- *   RSX_ETIMEOUT (the call's results are then invalid; the context stays usable).
+ * rsx_set_wait_limit: spin rounds a CTA of the context's Householder reductions waits
+ *   for the others before giving up (the grid-wide barrier of the cooperative form, 2^24
+ *   rounds by default; the messages of the register-resident cluster form, 2^22 polls by default
+ *   and at most; both far beyond any normal wait).  spins < 0 restores the defaults, 0 makes
+ *   every CTA (of the grid barrier: every CTA but the last arriver) give up at once.  When
+ *   one gives up, all leave at their next wait, the copies in flight are waited for, and
+ *   rsx_sync_status reports RSX_ETIMEOUT (the call's results are then invalid; the context
+ *   stays usable).
  * rsx_inject_fault: kind RSX_FAULT_ALLOC makes the workspace allocation after `after`
  *   more successful ones fail with RSX_ENOMEM without touching the device (once);
  *   RSX_FAULT_PIVOT makes the next rsx_ace_build factorise the ACE matrix with its sign

@@ -854,7 +854,8 @@ static int tridiagonalise(rsx_ctx* c, F* A, int n, F* d, F* e, F* tau, F* scr, F
       cudaGetLastError();
       return -1;
     }
-    return check_cuda(c, cudaLaunchKernelEx(&cfg, kern, A, n, d, e, tau, c->status), "cluster tridiagonalisation");
+    const uint32_t limit = c->wait_limit < 0 ? kTridiagWaitLimit : (uint32_t)std::min<long long>(c->wait_limit, kTridiagWaitLimit);
+    return check_cuda(c, cudaLaunchKernelEx(&cfg, kern, A, n, d, e, tau, limit, c->status), "cluster tridiagonalisation");
   };
   if constexpr (sizeof(F) == 4) {
     if (force.empty() && n >= 64) {

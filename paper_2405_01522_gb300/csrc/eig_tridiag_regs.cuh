@@ -58,10 +58,11 @@ struct TridiagRegs {
     float vav[W];            // shares of v^T A22 v
     uint64_t bar[2];
     int abort;
+    int last;                // step whose messages this CTA sent last
   };
 };
 
-constexpr uint32_t kTridiagWaitLimit = 1u << 22;   // try_wait rounds (each suspends for a while)
+constexpr uint32_t kTridiagWaitLimit = 1u << 22;   // try_wait rounds (each suspends for a while); 0: no waiting at all
 
 __device__ __forceinline__ uint32_t peer_smem(const void* p, int rank) {
   uint32_t a;
@@ -108,6 +109,11 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
   return ok != 0;
 }
 
+// bytes that no sender will complete any more, taken off the current phase's count
+__device__ __forceinline__ void mbar_complete_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(tc::smem_u32(bar)), "r"(bytes) : "memory");
+}
+
 // Sums of N values per lane over the warp's lanes: N = 2^b values leave row (lane >> (5 - b)) in x[0].
 template <int N>
 __device__ __forceinline__ void warp_row_sums(float (&x)[N], int lane) {
@@ -127,7 +133,7 @@ __device__ __forceinline__ void warp_row_sums(float (&x)[N], int lane) {
 template <int NL>
 __global__ void __launch_bounds__(TridiagRegs<NL>::NT, 1)
     k_tridiag_regs(float* __restrict__ A, int n, float* __restrict__ d, float* __restrict__ e,
-                   float* __restrict__ tau, int* __restrict__ status) {
+                   float* __restrict__ tau, uint32_t wait_limit, int* __restrict__ status) {
   using T = TridiagRegs<NL>;
   constexpr int CS = T::CS, RG = T::RG, CG = T::CG, NR = T::NR, W = T::W, NT = T::NT, NC = T::NC;
   constexpr int NB = NR < 8 ? NR : 8;   // rows summed together
@@ -199,7 +205,8 @@ __global__ void __launch_bounds__(TridiagRegs<NL>::NT, 1)
       }
     }
   };
-  for (int k = 0; k + 2 < n; ++k) {
+  int k = 0;
+  for (; k + 2 < n; ++k) {
     const int m0 = k + 1, b = k & 1;
     const float* col = sm.col[b];
     if (tid == 0) tc::mbar_arrive_expect_tx(&sm.bar[b], T::kBytes);
@@ -317,8 +324,8 @@ __global__ void __launch_bounds__(TridiagRegs<NL>::NT, 1)
     const uint32_t phase = (uint32_t)(k >> 1) & 1u;
     {
       uint32_t tries = 0;
-      while (live && !mbar_try_wait_cluster(&sm.bar[b], phase))
-        if (++tries > kTridiagWaitLimit || *(volatile int*)&sm.abort) {
+      while (live && (wait_limit == 0 || !mbar_try_wait_cluster(&sm.bar[b], phase)))
+        if (++tries > wait_limit || *(volatile int*)&sm.abort) {
           sm.abort = 1;
           live = false;
         }
@@ -359,6 +366,8 @@ __global__ void __launch_bounds__(TridiagRegs<NL>::NT, 1)
     }
   }
   if (live && n > 2) update(n - 3);
+  const int last = live ? n - 3 : k;
+  if (tid == 0) sm.last = last;
   if (!live && tid == 0 && status) atomicMax(status, RSX_ETIMEOUT);
   // diagonal, last subdiagonal
 #pragma unroll
@@ -371,6 +380,26 @@ __global__ void __launch_bounds__(TridiagRegs<NL>::NT, 1)
       if (i == n - 1 && j == n - 2) e[n - 2] = x;
     }
   if (me == 0 && tid == 0 && n >= 3) tau[n - 2] = 0.f;
+  cl.sync();   // every message has been sent
+  // A CTA that gave up at step `last` (n >= 3 then) waits for the messages on their way to it: those
+  // of this step from the CTAs that reached it, and of the next from those that passed it (nobody
+  // sends step last + 2's without this CTA's of last + 1; everybody sent last - 1's).
+  if (!live && warp == 0) {
+    const int theirs = lane < CS ? *cl.map_shared_rank(&sm.last, lane) : -1;
+    const uint32_t here = __popc(__ballot_sync(0xffffffffu, theirs >= last));
+    const uint32_t next = __popc(__ballot_sync(0xffffffffu, theirs > last));
+    if (lane == 0) {
+      constexpr uint32_t bytes = T::kBytes / CS;   // of one CTA's message
+      uint64_t *b0 = &sm.bar[last & 1], *b1 = &sm.bar[(last & 1) ^ 1];
+      if (here < CS) mbar_complete_tx(b0, (CS - here) * bytes);
+      if (next > 0) tc::mbar_arrive_expect_tx(b1, next * bytes);
+      for (uint32_t i = 0; i < kTridiagWaitLimit && !mbar_try_wait_cluster(b0, (uint32_t)(last >> 1) & 1u); ++i) {
+      }
+      for (uint32_t i = 0; next > 0 && i < kTridiagWaitLimit && !mbar_try_wait_cluster(b1, (uint32_t)((last + 1) >> 1) & 1u); ++i) {
+      }
+    }
+    __syncwarp();
+  }
   cl.sync();   // no CTA leaves while others may still address its shared memory
 }
 }  // namespace rsx
