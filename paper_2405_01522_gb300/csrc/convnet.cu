@@ -711,11 +711,9 @@ struct rsx_net {
   float* adam_m = nullptr;
   float* adam_v = nullptr;
   unsigned char* wimg = nullptr;   // weight images of the five convolutions (k_pack_weights)
-  float* act = nullptr;      // relu(z1), relu(z2): packed planes, 16 floats' bytes per voxel each
-  size_t act_elems = 0;
-  float* gout = nullptr;     // packed planes of x, dy, d z1, d z2, and the FP32 output
-  size_t gout_elems = 0;
-  float* part = nullptr;
+  float* act = nullptr;      // packed planes, 16 floats' bytes per voxel each: relu(z1), relu(z2), and two
+  size_t act_elems = 0;      // more for the gradients (backward)
+  float* part = nullptr;     // partial sums
   size_t part_elems = 0;
   double* loss = nullptr;
   int* status = nullptr;     // device status word (RSX_ETIMEOUT from a bounded wait)
@@ -845,22 +843,25 @@ int forward(rsx_net* n, const float* x, int B, int D, int H, int W, float* out, 
 
 // gradients of the masked MSE loss w.r.t. all parameters into n->grads; loss (device double) += value
 int backward(rsx_net* n, const float* x, const float* target, int B, int D, int H, int W, int border, cudaStream_t s) {
+  // Device memory is what limits a training batch: four sets of planes, 64 floats a voxel.  Each
+  // holds what is alive in turn (in stream order): a2 then the partial sums of layer 2's weight
+  // gradient, which may run on into gy's, then d z1; gy then x's planes; y then d z2.
   const size_t vol = (size_t)D * H * W, planes = (size_t)B * kC2 * vol;   // floats' worth of one set of planes
-  int rc = ngrow(n, &n->gout, &n->gout_elems, 4 * planes + (size_t)B * vol);
+  int rc = ngrow(n, &n->act, &n->act_elems, 4 * planes);
   if (rc) return rc;
   const int nwg = ((W + kWgX - 1) / kWgX) * ((H + kWgY - 1) / kWgY) * ((D + kWgZ - 1) / kWgZ);
   const int ncv = conv_blocks(D, H, W);
-  const size_t wpart = (size_t)B * nwg * kW2, bpart = std::max((size_t)B * ncv * 16, (size_t)kMseBlocks);
+  const size_t wpart2 = (size_t)B * nwg * kW2, bpart = std::max((size_t)B * ncv * 16, (size_t)kMseBlocks);
+  const bool in_planes = wpart2 <= 2 * planes;   // not so only in boxes of a few voxels
+  const size_t wpart = in_planes ? (size_t)B * nwg * std::max(kW1, kW3) : wpart2;
   rc = ngrow(n, &n->part, &n->part_elems, wpart + bpart);
   if (rc) return rc;
-  float *xp = n->gout, *gy = xp + planes, *g2 = gy + planes, *g1 = g2 + planes, *y = g1 + planes;
+  float *a1 = n->act, *a2 = a1 + planes, *gy = a2 + planes, *g2 = gy + planes;
+  float *part2 = in_planes ? a2 : n->part, *g1 = a2, *xp = gy, *y = g2;
   float* bp = n->part + wpart;
   rc = pack_weights(n, true, s);
-  if (!rc) rc = forward_layers(n, x, B, D, H, W, y, s);   // (re)sizes n->act
+  if (!rc) rc = forward_layers(n, x, B, D, H, W, y, s);
   if (rc) return rc;
-  float* a1 = n->act;
-  float* a2 = n->act + planes;
-  k_pack_planes<kC1><<<1024, 256, 0, s>>>(x, B, D, H, W, (uint4*)xp);
   k_mse<<<kMseBlocks, 256, 0, s>>>(y, target, (uint4*)gy, B, D, H, W, border, n->loss, bp);
   k_part_reduce<<<1, 32 * kRedWarps, 0, s>>>(bp, kMseBlocks, kC4, 0, n->grads + kOffB3);
   rc = ncuda(n, cudaGetLastError(), "loss");
@@ -882,10 +883,11 @@ int backward(rsx_net* n, const float* x, const float* target, int B, int D, int 
   if (!rc) rc = conv<kInPlanes, kOutMask>(n, gy, dgrad(kImgD3, g2, a2), "data gradient 3", s);
   if (!rc) k_part_reduce<<<1, 32 * kRedWarps, 0, s>>>(bp, B * ncv, kC3, 0, n->grads + kOffB2);
   // layer 2
-  if (!rc) rc = wgrad<kC2, kC3>(n, a1, g2, n->part, nwg, B, D, H, W, n->grads + kOffW2, s);
+  if (!rc) rc = wgrad<kC2, kC3>(n, a1, g2, part2, nwg, B, D, H, W, n->grads + kOffW2, s);
   if (!rc) rc = conv<kInPlanes, kOutMask>(n, g2, dgrad(kImgD2, g1, a1), "data gradient 2", s);
   if (!rc) k_part_reduce<<<1, 32 * kRedWarps, 0, s>>>(bp, B * ncv, kC2, 0, n->grads + kOffB1);
   // layer 1
+  if (!rc) k_pack_planes<kC1><<<1024, 256, 0, s>>>(x, B, D, H, W, (uint4*)xp);
   if (!rc) rc = wgrad<kC1, kC2>(n, xp, g1, n->part, nwg, B, D, H, W, n->grads + kOffW1, s);
   return rc ? rc : ncuda(n, cudaGetLastError(), "network backward");
 }
@@ -1005,7 +1007,7 @@ int rsx_net_destroy(rsx_net* n) {
   if (!n) return RSX_OK;
   cudaSetDevice(n->device);
   cudaDeviceSynchronize();
-  void* bufs[] = {n->params, n->grads, n->adam_m, n->adam_v, n->wimg, n->act, n->gout, n->part, n->loss, n->status};
+  void* bufs[] = {n->params, n->grads, n->adam_m, n->adam_v, n->wimg, n->act, n->part, n->loss, n->status};
   for (void* p : bufs)
     if (p) cudaFree(p);
   delete n;
