@@ -96,9 +96,9 @@ int rsx_get_tuning(rsx_ctx* ctx, rsx_tuning* out);
 int rsx_set_tuning_ex(rsx_ctx* ctx, const rsx_tuning* t);
 /* Autotuner (the paper has no counterpart; a performance knob).  Times the exchange
  * apply for nocc x npsi pairs on synthetic device data under candidate knobs, by
- * coordinate descent from the current ones: the pass-1 block order (0, 4, 16, 64, all), then
- * output orbitals per chunk (1, 2, 4, all); applies the fastest to the context.  With a non-empty cache_path the result is appended
- * to that text file, keyed by box, precision, nocc, npsi, SM count and device name, and a
+ * coordinate descent from the current ones: p2_global 0 (where it is 1), the pass-1 block order
+ * (0, 4, 16, 64, all), then output orbitals per chunk (1, 2, 4, all); applies the fastest to
+ * the context.  With a non-empty cache_path the result is appended to that text file, keyed by box, precision, nocc, npsi, SM count and device name, and a
  * later call with the same key applies it without timing.  chosen (may be NULL) receives
  * the knobs, best_ms the best time (-1 if taken from the cache).  Synchronises the device.
  * Errors: RSX_EINVAL, RSX_ENOMEM. */

@@ -7,8 +7,8 @@
 //     a chunk's pair intermediates near L2 size between the passes, large chunks launch
 //     fewer, fuller grids).
 // The y/z pass has one kernel per edge and precision (poisson_pass2.cuh), so p2_threads and
-// p2_lanes choose nothing; p2_global (the work plane in global scratch) stays as the caller
-// set it: it measured three times slower wherever shared memory holds the plane.
+// p2_lanes choose nothing; p2_global = 1 (the work plane in global scratch) is only left, never
+// taken up: it measured three times slower wherever shared memory holds the plane.
 // The search is coordinate descent from the current knobs, each candidate timed on the
 // exchange apply of synthetic orbitals on the device (one warm-up, best of two runs, CUDA
 // events).  The winner is applied to the context and appended to a text cache keyed by
@@ -39,11 +39,13 @@ __global__ void k_fill_synthetic(R* x, size_t n, uint32_t seed) {
   }
 }
 
+// The leading tag changes with the kernels that the knobs were timed on: entries of other
+// versions are not looked at (rsx3: p2_global, block orders and chunks of earlier passes).
 std::string cache_key(const rsx_ctx* c, int nocc, int npsi) {
   cudaDeviceProp prop;
   cudaGetDeviceProperties(&prop, c->device);
   char buf[512];
-  snprintf(buf, sizeof(buf), "rsx3 %d %d %d %s %d %d %d %s", c->g.nz, c->g.ny, c->g.nx,
+  snprintf(buf, sizeof(buf), "rsx4 %d %d %d %s %d %d %d %s", c->g.nz, c->g.ny, c->g.nx,
            c->precision == RSX_FP32 ? "fp32" : "fp64", nocc, npsi, c->nsm, prop.name);
   for (char* p = buf; *p; ++p)
     if (*p == '\n' || *p == '|') *p = ' ';
@@ -190,14 +192,20 @@ extern "C" int rsx_autotune_ex(rsx_ctx* c, int nocc, int npsi, const char* cache
         best = t;
       }
     };
-    // 1. pass-1 block order
+    // 1. the work plane back in shared memory, if the caller left it in global scratch
+    if (best.p2_global) {
+      rsx_tuning t = best;
+      t.p2_global = 0;
+      consider(t);
+    }
+    // 2. pass-1 block order
     const int groups[5] = {0, 4, 16, 64, 1 << 30};
     for (int gi = 0; gi < 5; ++gi) {
       rsx_tuning t = best;
       t.p1_group = groups[gi];
       consider(t);
     }
-    // 2. output orbitals per chunk
+    // 3. output orbitals per chunk
     const int chs[4] = {1, 2, 4, 0};
     for (int b = 0; b < 4; ++b) {
       if (chs[b] >= npsi) continue;
