@@ -792,10 +792,11 @@ static int tridiagonalise(rsx_ctx* c, F* A, int n, F* d, F* e, F* tau, F* scr, F
   int gcap = sizeof(F) == 4 ? c->nsm : 64;
   if (const char* ev = getenv("RSX_TRIDIAG_CTAS")) gcap = std::max(1, atoi(ev));
   const int G = std::min(std::min(std::min(c->nsm * std::max(per_sm, 0), gcap), std::max(1, n / 2)), 1024);
-  // rows in distributed shared memory (16 CTAs, else 8), else the cooperative grid, else
-  // one 16-CTA cluster with the rows in global memory (slower than the grid at n ~ 1000,
-  // measured), else one CTA.  RSX_TRIDIAG_PATH = cluster, coop, global or cta forces one
-  // (tests cover every path with it).
+  // rows in registers (FP32, n <= 768), else in distributed shared memory (16 CTAs, else 8), else
+  // the cooperative grid, else one 16-CTA cluster with the rows in global memory (slower than
+  // the grid at n ~ 1000, measured), else one CTA.  RSX_TRIDIAG_PATH = regs, cluster, coop,
+  // global or cta forces one (tests cover every path with it); an FP32 reduction that the
+  // forced path does not serve is refused.
   const char* fp = getenv("RSX_TRIDIAG_PATH");
   const std::string force = fp ? fp : "";
   auto try_cluster = [&](int CS, bool grows) -> int {   // -1: not possible here
@@ -858,7 +859,7 @@ static int tridiagonalise(rsx_ctx* c, F* A, int n, F* d, F* e, F* tau, F* scr, F
     return check_cuda(c, cudaLaunchKernelEx(&cfg, kern, A, n, d, e, tau, limit, c->status), "cluster tridiagonalisation");
   };
   if constexpr (sizeof(F) == 4) {
-    if (force.empty() && n >= 64) {
+    if ((force.empty() || force == "regs") && n >= 64) {
       int r = -1;
       if (n <= 256)
         r = try_regs(std::integral_constant<int, 16>{});
