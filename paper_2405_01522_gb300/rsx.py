@@ -136,11 +136,17 @@ def _ptr(t):
     return ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p(0)
 
 
+# The current stream's handle without building a Stream object (3 us of a 20 us call).  A private
+# name of torch: None where it is missing, and the public way is taken.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     if stream is not None:
         return ctypes.c_void_p(stream.cuda_stream)
-    # the current stream's handle without building a Stream object (3 us of a 20 us call)
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    if _raw_stream is not None:
+        return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
+    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
 class Context:
