@@ -132,10 +132,10 @@ DFT_FLOPS = {1: 0, 2: 4, 3: 18, 4: 16, 5: 52, 6: 48, 7: 102, 8: 60, 10: 124, 12:
              24: 3 * 60 + 8 * 18}
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12     # SMs x FP32 lanes x FMA x max SM clock
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of the same
-# kernels: pass 2 on the full 512-pair launch at 96^3 (a one-pass metric set: 3.669 + 3.602
-# GB); the SYRK on a small case scaled by the panel bytes it reads
-PASS2_DRAM_BYTES_PER_PAIR_96 = 7.271e9 / 512
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of these
+# kernels: k_pass2<float, 12, 1> on the full 512-pair launch at 96^3 (a one-pass metric set: 3.67 + 3.61
+# GB, profiles/line_passes_96cubed.md); the SYRK on a small case scaled by the panel bytes it reads
+PASS2_DRAM_BYTES_PER_PAIR_96 = 7.28e9 / 512
 SYRK_DRAM_PER_PANEL_BYTE = 1.938e9 / 1.850e9    # DRAM bytes per byte of the two bf16 panels
 
 
@@ -338,8 +338,8 @@ def run_rsx(args, rank, local_rank, world):
     top = next(iter(kernels))
     roof = None
     if top in per_launch_pairs:
-        # the FFT passes are instruction-issue / FP32 bound (ncu: DRAM ~7%, issue ~60%):
-        # report the ALU roofline, with the HBM view alongside
+        # pass 2 is bound on the SM, not by HBM (ncu, 64 pairs: L1 data pipe 76%, issue 49%, FMA pipe
+        # 35%, DRAM 17%): report the ALU roofline, with the HBM view alongside
         byts = [algorithmic_bytes(top, shape, nq, NOCC, NPSI if nq == SOLVES_EXCHANGE else 0)
                 for nq in per_launch_pairs[top]]
         flops = [algorithmic_flops(top, shape, nq, 0) for nq in per_launch_pairs[top]]
@@ -358,7 +358,7 @@ def run_rsx(args, rank, local_rank, world):
                 "unit": "TFLOP/s", "frac": round(ach_f / FP32_PEAK_TFLOPS, 4), "traffic": traffic,
                 "traffic_source": (f"ncu DRAM bytes of the 512-pair launch ({per_pair / 1e6:.1f} MB per pair) times "
                                    "the average pairs per launch") if traffic else
-                                  "none: no capture of this kernel build yet",
+                                  "none: pass 2 was captured at 96^3 only",
                 "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 (FMA) x 2.07 GHz",
                 "algorithmic_flops_per_launch": avg_flops,
                 "hbm_view": {"achieved_gbs": round(ach_b, 1), "peak_gbs": hbm_peak, "frac": round(ach_b / hbm_peak, 4),
