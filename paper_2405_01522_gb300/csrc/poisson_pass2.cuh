@@ -10,7 +10,8 @@ namespace rsx {
 // divisor of the edge, so that every line has the same rows and columns), CTAs per SM asked of
 // the compiler, and the 8-row groups of a line's scratch held at a time.  FP32, us per pair at
 // 128 pairs: several CTAs per SM cover each other's barriers where the planes fit (A = 8: 2.87
-// as 2 x 256 threads, 3.10 as 1 x 512; A = 7: 2.21 at 2 x 224, 2.51 at 3 x 224, which spills);
+// as 2 x 256 threads, 3.10 as 1 x 512; A = 7: 2.21 at 2 x 224, 2.51 at 3 x 224, which spills;
+// A = 6 at 3 CTAs spills 44 bytes, A = 4 4 bytes; fewer CTAs were not measured there);
 // at A = 12 the plane allows one CTA and 48 lines (12 warps) beat 32 once the scratch holds one
 // group (10.08 us; 10.42 at 32 lines, 11.14 with all three groups in scratch).
 template <typename R>

@@ -7,9 +7,9 @@
 
 namespace rsx {
 
-// Lines per CTA (8 lanes each) and CTAs per SM asked of the compiler.  Without the z inverse the
-// transforms need fewer registers than pass 2's, so A = 14 runs on 8 lanes here (56 lines: 16.1 us per
-// transition at 112^3, 36 at 28 lines; 20.6 for 16 lanes x A).
+// Lines per CTA (8 lanes each) and CTAs per SM asked of the compiler.  Without the z inverse A = 14
+// pays on 8 lanes here: 56 lines (128 registers a thread, 416 bytes of spill stores) take 16.1 us
+// per transition at 112^3, 28 lines 36; 16 lanes x A took 20.6.
 __host__ __device__ constexpr int spec_lines(int A) { return A == 14 ? 56 : A == 10 ? 40 : p2_lines<float>(A); }
 __host__ __device__ constexpr int spec_min_ctas(int A) { return p2_min_ctas<float>(A); }
 __host__ __device__ constexpr int spec_pitch(int A) { return 16 * A + 2; }   // as p2_pitch on 8 lanes
