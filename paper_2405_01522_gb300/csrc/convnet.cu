@@ -275,10 +275,13 @@ __global__ void __launch_bounds__(cv_threads(IN), 2) k_conv(const __grid_constan
     }
     // no copy or arrival may land after the CTA exits: the weights, then the last commit of every
     // barrier (bounded waits; after a time-out at plane p, ready[p] closes what came before it)
-    for (uint32_t k = 0; k < kWaitLimit && !mbar_try_wait(&wbar, 0); ++k) {
+    int last = np - 1;
+    if (!ok) {
+      for (uint32_t k = 0; k < kWaitLimit && !mbar_try_wait(&wbar, 0); ++k) {
+      }
+      last = p > 0 ? p : -1;
+      if (last >= 0 && lead) mma_commit(&ready[last]);
     }
-    const int last = ok ? np - 1 : (p > 0 ? p : -1);
-    if (!ok && last >= 0 && lead) mma_commit(&ready[last]);
     for (int i = max(0, n - kCvSlots); i < n; ++i)
       for (uint32_t k = 0; k < kWaitLimit && !mbar_try_wait(&empty[i % kCvSlots], (uint32_t)((i / kCvSlots) & 1)); ++k) {
       }
